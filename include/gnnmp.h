@@ -281,7 +281,8 @@ typedef struct gnn_mp_params {
     gnn_mlp node;
 } gnn_mp_params;
 
-#define GNN_PREC_FP32 0   /* plain FP32 SIMT kernels, FP32 edge state                       */
+#define GNN_PREC_FP32 0   /* FP32 states, weights, sums and results: tensor-core Linears on
+                             exact three-way BF16 splits up to H = 128, SIMT kernels above  */
 #define GNN_PREC_BF16 1   /* fused tcgen05 kernels: BF16 GEMM operands, FP32 accumulation,
                              FP32 sums/LayerNorm statistics, BF16 edge state and edge grads */
 #define GNN_HALO_SYNC 0   /* consistent layer (Eq. 5c-5d applied)                           */
@@ -513,7 +514,7 @@ int gnn_profile_report(char* out, size_t bytes);
  * with the library's own FMA kernel (independent chains of fused multiply-adds
  * per thread, two blocks of 1024 threads per SM, best of three CUDA-event timed
  * launches after one warm-up), in TFLOP/s at 2 FLOPs per FMA, and its SM count.
- * It is the peak the plain FP32 SIMT path is measured against. Synchronous on
+ * It is the peak that SIMT FP32 kernels are measured against. Synchronous on
  * `stream`; allocates nothing.
  *
  * gnn_selftest_bounded_wait: launches one warp that waits on an mbarrier no

@@ -1,6 +1,6 @@
 // Diagnostics of libgnnmp with no counterpart in the paper:
-//   * the FP32 FMA throughput of the device, the peak the plain FP32 SIMT path
-//     is measured against (a long chain of independent fused multiply-adds per
+//   * the FP32 FMA throughput of the device, the peak that SIMT FP32 kernels
+//     are measured against (a long chain of independent fused multiply-adds per
 //     thread, CUDA-event timed);
 //   * a self-test of the bounded device-side waits: a kernel waits on an
 //     mbarrier that no thread ever arrives at, with a caller-given limit, and

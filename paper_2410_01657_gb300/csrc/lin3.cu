@@ -1,0 +1,1059 @@
+// FP32 Linear layers on the tensor cores, for the FP32 path's MLPs.
+//
+// An FP32 number has 24 significant bits, so it is exactly the sum of three
+// BF16 numbers of 8 bits each: hi = x rounded to BF16, mid = x - hi rounded,
+// lo = the rest (both differences are exact). A product x w is then the sum of
+// nine BF16 products, each exact in FP32; the six largest are accumulated in
+// FP32 by tcgen05.mma and the three left out (mid lo, lo mid, lo lo) are below
+// 2^-25 |x w|, of either sign. (Splitting by clearing bits costs the same but
+// makes every piece agree in sign with x: the parts left out then add up.)
+// The tensor core truncates its running sums, so a sum must not carry terms
+// far below it: the hi hi products have an accumulator of their own, the five
+// small ones share another, and the epilogue adds the two. Sums in tensor
+// memory run over at most 256 products per output (inputs) or one tile of rows
+// (weight gradients, continued in FP32 registers, rounding to nearest).
+//
+// What bounds it: at width 64 a Linear moves 512 bytes per row for 49 kFLOP of
+// BF16 products, 96 FLOP per byte, far below the ridge: HBM, if the splitting
+// (about 6 instructions per element) and the epilogue are hidden. So the block
+// is specialised: eight warps load FP32 rows, split them and write the three
+// operand tiles (swizzled K-major rows); one thread issues the MMAs; two
+// groups of four warps take alternate tiles from two tensor-memory
+// accumulators, through a per-warp staging tile so that every global access of
+// an epilogue (bias, residual, gathers, stores) is a run of whole 64-byte
+// pieces of rows.
+
+#include <algorithm>
+
+#include "device_common.cuh"
+#include "fused_common.cuh"
+#include "lin3.h"
+#include "profiler.h"
+
+namespace gnn {
+namespace lin3 {
+
+using namespace tc;
+using fused::align_up;
+using fused::aligned_smem;
+using fused::desc_step;
+using fused::kmajor_off;
+using fused::span_of;
+
+cudaError_t take_device_error(unsigned int* out) { return take_device_error_word(out); }
+
+namespace {
+
+// k_lin3: 4 producer warps, 8 epilogue warps, one MMA warp: 13 warps leave each
+// thread 128 registers (at 17 it is 96), which the epilogue's operands need.
+// k_wgrad3: two operands to split and little to do at the end, 8 + 8 + 1 warps.
+constexpr int kProducers = 128, kEpilogue = 256;
+constexpr int kThreads = kProducers + kEpilogue + 32;
+constexpr int kProducerWarps = kProducers / 32, kEpilogueWarps = kEpilogue / 32;
+constexpr int kSide = 128;   // k_wgrad3: producer threads of one operand
+constexpr int kWThreads = 2 * kSide + kEpilogue + 32;
+constexpr int kWProducerWarps = 2 * kSide / 32;
+constexpr int kStageLd = 20;                      // floats per row of a 32 x 16 staging tile: 16-byte rows, no conflicts
+constexpr uint32_t kStageBytes = 32 * kStageLd * 4;
+constexpr uint32_t kSmemMax = 227 * 1024;
+
+__host__ __device__ inline int pad16(int n) { return (n + 15) / 16 * 16; }
+__host__ __device__ inline int pow2_width(int n) { return n <= 16 ? 16 : (n <= 32 ? 32 : (n <= 64 ? 64 : 128)); }
+__host__ __device__ inline uint32_t pow2_cols(uint32_t n) {
+    uint32_t c = 32;
+    while (c < n) c <<= 1;
+    return c;
+}
+
+// ------------------------------------------------------------------ device helpers
+
+// Eight FP32 values as three BF16 octets whose sum they are.
+__device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& mid, uint4& lo) {
+    uint32_t h[4], m[4], l[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float a = v[2 * i], b = v[2 * i + 1], x, y;
+        h[i] = pack_bf16x2(a, b);
+        unpack_bf16x2(h[i], x, y);
+        a -= x;
+        b -= y;
+        m[i] = pack_bf16x2(a, b);
+        unpack_bf16x2(m[i], x, y);
+        l[i] = pack_bf16x2(a - x, b - y);
+    }
+    hi = make_uint4(h[0], h[1], h[2], h[3]);
+    mid = make_uint4(m[0], m[1], m[2], m[3]);
+    lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// Up to n (may be <= 0) of the 8 values at p, the rest zero. VEC: p is 16-byte
+// aligned and n is a multiple of 4.
+template <bool VEC>
+__device__ __forceinline__ void load8(const float* p, int n, float* v) {
+    if constexpr (VEC) {
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 a = n > 0 ? __ldg(reinterpret_cast<const float4*>(p)) : z;
+        const float4 b = n > 4 ? __ldg(reinterpret_cast<const float4*>(p) + 1) : z;
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = i < n ? __ldg(p + i) : 0.f;
+    }
+}
+
+// Four values of a row, of which n exist (VEC: all four or none). The loads are
+// plain ones: an epilogue may read the buffer it writes (same lane, same address).
+template <bool VEC>
+__device__ __forceinline__ float4 load4(const float* p, int n) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (VEC) {
+        if (n > 0) v = *reinterpret_cast<const float4*>(p);
+    } else {
+        if (n > 0) v.x = p[0];
+        if (n > 1) v.y = p[1];
+        if (n > 2) v.z = p[2];
+        if (n > 3) v.w = p[3];
+    }
+    return v;
+}
+template <bool VEC>
+__device__ __forceinline__ void store4(float* p, int n, float4 v) {
+    if constexpr (VEC) {
+        if (n > 0) *reinterpret_cast<float4*>(p) = v;
+    } else {
+        if (n > 0) p[0] = v.x;
+        if (n > 1) p[1] = v.y;
+        if (n > 2) p[2] = v.z;
+        if (n > 3) p[3] = v.w;
+    }
+}
+__device__ __forceinline__ float4 add4(float4 a, float4 b) {
+    const float2 l = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+    const float2 h = __fadd2_rn(make_float2(a.z, a.w), make_float2(b.z, b.w));
+    return make_float4(l.x, l.y, h.x, h.y);
+}
+
+template <int V>
+struct Int {
+    static constexpr int value = V;
+};
+
+// One lane of the warp waits, the warp agrees (and is converged afterwards).
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int lane) {
+    int ok = 1;
+    if (lane == 0) ok = mbar_wait(bar, parity) ? 1 : 0;
+    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
+// 16 columns of the lane's row: the hi hi sum plus the small products' sum.
+__device__ __forceinline__ void load_sum16(uint32_t taddr, int NP, float* v) {
+    float u[16];
+    tmem_ld16(taddr, v);
+    tmem_ld16(taddr + NP, u);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {
+        const float2 w = __fadd2_rn(make_float2(v[i], v[i + 1]), make_float2(u[i], u[i + 1]));
+        v[i] = w.x;
+        v[i + 1] = w.y;
+    }
+}
+
+// ELU (alpha 1) of two values: z above zero, e^z - 1 at and below it, by the
+// usual two steps: Cody and Waite's reduction z = n ln 2 + r, |r| <= ln 2 / 2
+// (ln 2 in two parts, n by adding and subtracting 1.5 * 2^23), and Taylor's
+// series of e^r - 1 up to r^8 (the rest is below 6e-10 r); then
+// e^z - 1 = 2^n (e^r - 1) + (2^n - 1), exact in its last term for n >= -24. On
+// the packed FP32 pipe it is 12 instructions per value where a call of expm1f
+// is about 40. Below -87 it is -1; a NaN stays one (the select is on z <= 0).
+__device__ __forceinline__ float2 elu_pair(float2 z) {
+    const float2 c = make_float2(fmaxf(z.x, -87.f), fmaxf(z.y, -87.f));
+    auto both = [](float v) { return make_float2(v, v); };
+    const float2 t = __ffma2_rn(c, both(1.4426950408889634f), both(12582912.f));
+    const float2 n = __fadd2_rn(t, both(-12582912.f));
+    float2 r = __ffma2_rn(n, both(-0.693145751953125f), c);
+    r = __ffma2_rn(n, both(-1.4286068203094172e-6f), r);
+    float2 q = __ffma2_rn(r, both(1.f / 40320.f), both(1.f / 5040.f));
+    q = __ffma2_rn(q, r, both(1.f / 720.f));
+    q = __ffma2_rn(q, r, both(1.f / 120.f));
+    q = __ffma2_rn(q, r, both(1.f / 24.f));
+    q = __ffma2_rn(q, r, both(1.f / 6.f));
+    q = __ffma2_rn(q, r, both(0.5f));
+    q = __ffma2_rn(__fmul2_rn(q, r), r, r);
+    const float2 p2 = make_float2(__uint_as_float((__float_as_uint(t.x) << 23) + 0x3f800000u),
+                                  __uint_as_float((__float_as_uint(t.y) << 23) + 0x3f800000u));
+    const float2 e = __ffma2_rn(p2, q, __fadd2_rn(p2, both(-1.f)));
+    return make_float2(z.x <= 0.f ? e.x : z.x, z.y <= 0.f ? e.y : z.y);
+}
+
+// The six products of a split pair, smallest first: (term of A, term of B).
+__device__ constexpr int kTermA[6] = {2, 0, 1, 1, 0, 0};
+__device__ constexpr int kTermB[6] = {0, 2, 1, 0, 1, 0};
+
+// ------------------------------------------------------------------ shared memory
+
+struct Smem {
+    uint32_t w, a, stg, sums, par, bar, tm, total;
+    uint32_t wterm, aterm;
+};
+
+// W: nkb blocks x 3 terms of [NP x KB]; a: stages x 3 terms of [128 x KB].
+__host__ __device__ inline Smem lin_smem(int NP, int KB, int nkb, int stages) {
+    Smem s;
+    s.wterm = (uint32_t)NP * KB * 2;
+    s.aterm = 128u * KB * 2;
+    s.w = 0;
+    s.a = align_up((uint32_t)nkb * 3 * s.wterm, 1024);
+    s.stg = s.a + (uint32_t)stages * 3 * s.aterm;
+    s.sums = s.stg + kEpilogueWarps * kStageBytes;           // [8 warps][2 NP]
+    s.par = s.sums + kEpilogueWarps * 2 * (uint32_t)NP * 4;  // bias, gamma, beta
+    s.bar = align_up(s.par + 3 * (uint32_t)NP * 4, 8);       // full[4], empty[4], acc_full[2], acc_empty[2]
+    s.tm = s.bar + 12 * 8;
+    s.total = s.tm + 16 + 1024;
+    return s;
+}
+
+// ------------------------------------------------------------------ k_lin3
+
+// Producer warps: load FP32 rows (every block of W columns of every source),
+// split them, write the three operand tiles of a stage.
+template <int W, bool VEC, int MODE>
+__device__ __forceinline__ void lin_producer(const Args& A, const Smem& P, uint8_t* sm, uint64_t* full,
+                                             uint64_t* empty, int tid, int lane) {
+    constexpr int U = W / 8, RS = kProducers / U, IT = 128 / RS;   // pieces of 8 columns per row; rows per step; steps
+    constexpr int B = IT < 8 ? IT : 8;                             // pieces in flight per thread
+    constexpr int S = span_of(W);
+    static_assert((RS * S) % 1024 == 0, "the swizzle repeats every RS rows");
+    const int c = (tid % U) * 8, row0 = tid / U;
+    const uint32_t off0 = tile_off(row0, c, 128, S);
+    const int stages = A.stages, nkb = A.nkb[0] + A.nkb[1];
+    int st = 0, use = 0;
+    for (int t = blockIdx.x; t < A.n_tiles; t += gridDim.x) {
+        if (VEC && tid == 0 && t + (int)gridDim.x < A.n_tiles) {   // the next tile's rows into L2
+            const int64_t rn = (int64_t)(t + (int)gridDim.x) * 128;
+            const int64_t nr = std::min<int64_t>(128, A.rows - rn);
+            for (int s = 0; s < 2; ++s)
+                if (A.K[s] && A.lda[s] == A.K[s]) prefetch_l2(A.A[s] + rn * A.lda[s], (uint32_t)(nr * A.K[s] * 4));
+            if (A.add && A.ldadd == A.N) prefetch_l2(A.add + rn * A.N, (uint32_t)(nr * A.N * 4));
+            if (MODE == kLnAdjoint && A.g0) prefetch_l2(A.g0 + rn * A.N, (uint32_t)(nr * A.N * 4));
+        }
+        const int left = (int)std::min<int64_t>(128, A.rows - (int64_t)t * 128);
+        for (int b = 0; b < nkb; ++b) {
+            const int s = b < A.nkb[0] ? 0 : 1;
+            const int kc = (b - (s ? A.nkb[0] : 0)) * W + c;
+            const int nk = A.K[s] - kc;
+            const float* src = A.A[s] + ((int64_t)t * 128 + row0) * A.lda[s] + kc;
+            const int64_t step = RS * A.lda[s];
+            uint8_t* dst = sm + P.a + (uint32_t)st * 3 * P.aterm + off0;
+            const bool whole = left == 128 && A.K[s] % W == 0;
+#pragma unroll
+            for (int i0 = 0; i0 < IT; i0 += B) {
+                float v[B][8];
+                if (whole) {
+#pragma unroll
+                    for (int i = 0; i < B; ++i) load8<VEC>(src + (i0 + i) * step, 8, v[i]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < B; ++i)
+                        load8<VEC>(src + (i0 + i) * step, row0 + (i0 + i) * RS < left ? nk : 0, v[i]);
+                }
+                if (i0 == 0 && use > 0 && !warp_wait(empty + st, (uint32_t)(use - 1) & 1u, lane)) return;
+#pragma unroll
+                for (int i = 0; i < B; ++i) {
+                    uint4 h, m, l;
+                    split8(v[i], h, m, l);
+                    uint8_t* q = dst + (i0 + i) * RS * S;
+                    *reinterpret_cast<uint4*>(q) = h;
+                    *reinterpret_cast<uint4*>(q + 128 * S) = m;
+                    *reinterpret_cast<uint4*>(q + 2 * 128 * S) = l;
+                }
+            }
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full + st);
+            if (++st == stages) {
+                st = 0;
+                ++use;
+            }
+        }
+    }
+}
+
+// OPS: what an epilogue adds or needs of other rows: nothing, one row (add), or gathered rows
+// (P, Q of kElu; da, w of kLnAdjoint).
+enum Ops { kOpsNone = 0, kOpsRow, kOpsGather };
+
+template <int MODE, int OPS, bool VEC>
+__global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Args A) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* sm = aligned_smem(smem_raw);
+    const int NP = A.NP, KB = A.KB, S = span_of(KB), stages = A.stages, nkb = A.nkb[0] + A.nkb[1], N = A.N;
+    const Smem P = lin_smem(NP, KB, nkb, stages);
+    float* sPar = reinterpret_cast<float*>(sm + P.par);
+    uint64_t* full = reinterpret_cast<uint64_t*>(sm + P.bar);
+    uint64_t* empty = full + 4;
+    uint64_t* acc_full = full + 8;
+    uint64_t* acc_empty = full + 10;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + P.tm);
+    const uint32_t NCOLS = pow2_cols(4 * (uint32_t)NP);   // two tiles x {hi hi, small products}
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    if (warp == 0) {
+        tmem_alloc(tslot, NCOLS);
+        tmem_relinquish();
+    }
+    if (tid == 0) {
+        for (int i = 0; i < stages; ++i) {
+            mbar_init(full + i, kProducerWarps);
+            mbar_init(empty + i, 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(acc_full + i, 1);
+            mbar_init(acc_empty + i, 4);
+        }
+        fence_mbar_init();
+    }
+    {   // the weights, split, for the block's lifetime
+        const int upr = KB / 8, per = NP * upr;
+        for (int i = tid; i < nkb * per; i += kThreads) {
+            const int b = i / per, n = (i - b * per) / upr, k8 = (i % upr) * 8;
+            const int s = b < A.nkb[0] ? 0 : 1;
+            const int k0 = (b - (s ? A.nkb[0] : 0)) * KB + k8;
+            const bool second = n >= A.nsplit;
+            const float* w = A.W[s] + (second ? A.noff + (int64_t)(n - A.nsplit) * A.sn : (int64_t)n * A.sn);
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = (n < N && k0 + j < A.K[s]) ? __ldg(w + (k0 + j) * A.sk) : 0.f;
+            uint4 t[3];
+            split8(v, t[0], t[1], t[2]);
+            const uint32_t off = tile_off(n, k8, NP, S);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) *reinterpret_cast<uint4*>(sm + P.w + (b * 3 + j) * P.wterm + off) = t[j];
+        }
+        for (int i = tid; i < NP; i += kThreads) {
+            sPar[i] = (A.bias && i < N) ? A.bias[i] : 0.f;
+            if (MODE == kLayerNorm || MODE == kLnAdjoint) {
+                sPar[NP + i] = i < N ? A.gamma[i] : 0.f;
+                sPar[2 * NP + i] = i < N ? A.beta[i] : 0.f;
+            }
+        }
+        if (MODE == kLnAdjoint) {
+            float* z = reinterpret_cast<float*>(sm + P.sums);
+            for (int i = tid; i < kEpilogueWarps * 2 * NP; i += kThreads) z[i] = 0.f;
+        }
+    }
+    fence_proxy_async();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot;
+
+    if (warp < kProducerWarps) {
+        if (KB == 64) lin_producer<64, VEC, MODE>(A, P, sm, full, empty, tid, lane);
+        else if (KB == 32) lin_producer<32, VEC, MODE>(A, P, sm, full, empty, tid, lane);
+        else lin_producer<16, VEC, MODE>(A, P, sm, full, empty, tid, lane);
+    } else if (warp == kProducerWarps + kEpilogueWarps) {
+        // ---- one thread issues the MMAs
+        if (lane == 0) {
+            const uint32_t id = idesc_bf16(128, NP);
+            const uint64_t a0 = kmajor_desc(smem_u32(sm + P.a), 128, S, 0);
+            const uint64_t w0 = kmajor_desc(smem_u32(sm + P.w), NP, S, 0);
+            int n = 0, j = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++j) {
+                const int buf = j & 1;
+                const uint32_t d = tmem + (uint32_t)(buf * 2 * NP);
+                if (j >= 2) ok = mbar_wait(acc_empty + buf, (uint32_t)((j >> 1) - 1) & 1u);
+                for (int b = 0; b < nkb && ok; ++b, ++n) {
+                    const int st = n % stages, use = n / stages;
+                    ok = mbar_wait(full + st, (uint32_t)use & 1u);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t ao = (uint32_t)st * 3 * P.aterm, wo = (uint32_t)b * 3 * P.wterm;
+                    auto issue = [&](auto kb) {
+#pragma unroll
+                        for (int p = 0; p < 6; ++p) {
+                            const uint64_t ap = desc_step(a0, ao + kTermA[p] * P.aterm);
+                            const uint64_t wp = desc_step(w0, wo + kTermB[p] * P.wterm);
+#pragma unroll
+                            for (int k0 = 0; k0 < decltype(kb)::value; k0 += 16)   // one swizzle block, 32 bytes a step
+                                mma_bf16(p < 5 ? d + NP : d, desc_step(ap, k0 * 2), desc_step(wp, k0 * 2), id,
+                                         (b > 0 || (p > 0 && p < 5) || k0 > 0) ? 1u : 0u);
+                        }
+                    };
+                    if (KB == 64) issue(Int<64>());
+                    else if (KB == 32) issue(Int<32>());
+                    else issue(Int<16>());
+                    mma_commit(empty + st);
+                }
+                if (ok) mma_commit(acc_full + buf);
+            }
+            // the last stage's release has arrived before the block may end
+            if (ok && n > 0) mbar_wait(empty + (n - 1) % stages, (uint32_t)((n - 1) / stages) & 1u);
+        }
+        __syncwarp();
+    } else {
+        // ---- epilogue: group eg takes the tiles of accumulator eg. A warp has 32 rows; it reads
+        // the accumulator by rows (lane = row) and everything else by pieces of 8 rows x 16 columns
+        const int ew = warp - kProducerWarps, eg = ew >> 2, q = ew & 3;
+        float* stg = reinterpret_cast<float*>(sm + P.stg + ew * kStageBytes);
+        float* sums = reinterpret_cast<float*>(sm + P.sums) + ew * 2 * NP;
+        const uint32_t tacc = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(eg * 2 * NP);
+        const int rs = lane >> 2, c4 = (lane & 3) * 4;
+        constexpr bool kGather = MODE == kElu && OPS == kOpsGather, kEdge = MODE == kLnAdjoint && OPS == kOpsGather;
+        bool ok = true;
+        int j = 0;
+        for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++j) {
+            if ((j & 1) != eg) continue;
+            const int64_t rb = (int64_t)t * 128 + 32 * q;
+            const int nv = (int)std::min<int64_t>(32, std::max<int64_t>(0, A.rows - rb));
+            // this lane's rows (clamped to the last one: loads need no test, stores have it) and their
+            // receivers, senders and weights
+            int64_t row[4];
+            int rv[4] = {0, 0, 0, 0}, sv[4] = {0, 0, 0, 0};
+            float wv[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                row[i] = nv > 0 ? rb + std::min(8 * i + rs, nv - 1) : 0;
+                if (kGather || kEdge) rv[i] = A.recv[row[i]];
+                if (kGather) sv[i] = A.snd[row[i]];
+                if (kEdge) wv[i] = A.w[row[i]];
+            }
+            // operands of one piece of the four rows
+            auto load_ops = [&](int c0, float4* x, float4* y) {
+                const int nc = N - (c0 + c4), col = VEC ? std::min(c0 + c4, N - 4) : c0 + c4;
+                (void)y;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if constexpr (kGather) {
+                        x[i] = load4<VEC>(A.P + (int64_t)rv[i] * A.ldpq + col, VEC ? 4 : nc);
+                        y[i] = load4<VEC>(A.Q + (int64_t)sv[i] * A.ldpq + col, VEC ? 4 : nc);
+                    } else if constexpr (MODE != kLnAdjoint && OPS == kOpsRow) {
+                        x[i] = load4<VEC>(A.add + row[i] * A.ldadd + col, VEC ? 4 : nc);
+                    }
+                }
+            };
+            // the upstream gradient of one piece of the four rows: formed (and, for edges, written by the
+            // same lane, perhaps over g0), then read again
+            auto load_g = [&](int c0, bool again, float4* g) {
+                const int nc = N - (c0 + c4), col = VEC ? std::min(c0 + c4, N - 4) : c0 + c4;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) g[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                const float* src = kEdge && again ? A.g_out : A.g0;
+                if (src) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) g[i] = load4<VEC>(src + row[i] * N + col, VEC ? 4 : nc);
+                }
+                if (kEdge && !again) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 d = load4<VEC>(A.da + (int64_t)rv[i] * N + col, VEC ? 4 : nc);
+                        g[i] = make_float4(g[i].x + wv[i] * d.x, g[i].y + wv[i] * d.y, g[i].z + wv[i] * d.z,
+                                           g[i].w + wv[i] * d.w);
+                    }
+                }
+            };
+            float4 x[4], y[4];
+            load_ops(0, x, y);   // before the wait: the first piece's operands
+            ok = warp_wait(acc_full + eg, (uint32_t)(j >> 1) & 1u, lane);
+            if (!ok) break;
+            tc_fence_after();
+            float mean = 0.f, rstd = 0.f, m1 = 0.f, m2 = 0.f;
+            if constexpr (MODE == kLayerNorm || MODE == kLnAdjoint) {
+                // row statistics: the lane's row, two passes over the accumulator
+                float s4[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int c0 = 0; c0 < N; c0 += 16) {
+                    float v[16];
+                    load_sum16(tacc + c0, NP, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) s4[i & 3] += v[i] + sPar[c0 + i];   // padding columns are zero
+                }
+                mean = ((s4[0] + s4[1]) + (s4[2] + s4[3])) / N;
+                float q4[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int c0 = 0; c0 < N; c0 += 16) {
+                    float v[16];
+                    load_sum16(tacc + c0, NP, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const float d = c0 + i < N ? v[i] + sPar[c0 + i] - mean : 0.f;
+                        q4[i & 3] = fmaf(d, d, q4[i & 3]);
+                    }
+                }
+                rstd = rsqrtf(((q4[0] + q4[1]) + (q4[2] + q4[3])) / N + A.eps);
+            }
+            if constexpr (MODE == kLnAdjoint) {
+                // g, and its two row sums against gamma and gamma * xhat
+                for (int c0 = 0; c0 < N; c0 += 16) {
+                    const int col = c0 + c4, nc = N - col;
+                    float4 g[4];
+                    load_g(c0, false, g);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int r = 8 * i + rs;
+                        if (kEdge && r < nv) store4<VEC>(A.g_out + row[i] * N + col, nc, g[i]);
+                        *reinterpret_cast<float4*>(stg + r * kStageLd + c4) = g[i];
+                    }
+                    float v[16];
+                    load_sum16(tacc + c0, NP, v);
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 16; i += 4) {
+                        const float4 g4 = *reinterpret_cast<const float4*>(stg + lane * kStageLd + i);
+                        const float gg[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            // (a clamped piece past the last column repeats real values: not counted)
+                            const float d = c0 + i + k < N ? __fmul_rn(gg[k], sPar[NP + c0 + i + k]) : 0.f;
+                            m1 += d;
+                            m2 = fmaf(d, (v[i + k] + sPar[c0 + i + k] - mean) * rstd, m2);
+                        }
+                    }
+                    __syncwarp();
+                }
+                m1 /= N;
+                m2 /= N;
+            }
+            for (int c0 = 0; c0 < NP; c0 += 16) {
+                const int col = c0 + c4, nc = N - col;
+                float v[16];
+                load_sum16(tacc + c0, NP, v);
+                if constexpr (MODE == kLayerNorm || MODE == kLnAdjoint) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] = (v[i] + sPar[c0 + i] - mean) * rstd;   // xhat
+                }
+#pragma unroll
+                for (int i = 0; i < 16; i += 4)
+                    *reinterpret_cast<float4*>(stg + lane * kStageLd + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                const float4 b = *reinterpret_cast<const float4*>(sPar + col);
+                float4 ga = b, be = b;
+                if constexpr (MODE == kLayerNorm || MODE == kLnAdjoint) {
+                    ga = *reinterpret_cast<const float4*>(sPar + NP + col);
+                    be = *reinterpret_cast<const float4*>(sPar + 2 * NP + col);
+                }
+                if constexpr (MODE == kLnAdjoint) load_g(c0, true, x);
+                __syncwarp();
+                float4 u[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) u[i] = *reinterpret_cast<const float4*>(stg + (8 * i + rs) * kStageLd + c4);
+                if constexpr (MODE == kElu) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        u[i] = add4(u[i], b);
+                        if constexpr (OPS == kOpsRow) u[i] = add4(u[i], x[i]);
+                        if constexpr (OPS == kOpsGather) u[i] = add4(u[i], add4(x[i], y[i]));
+                    }
+                } else if constexpr (MODE == kLayerNorm) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        u[i] = make_float4(u[i].x * ga.x + be.x, u[i].y * ga.y + be.y, u[i].z * ga.z + be.z,
+                                           u[i].w * ga.w + be.w);
+                        if constexpr (OPS == kOpsRow) u[i] = add4(u[i], x[i]);
+                    }
+                } else if constexpr (MODE == kLnAdjoint) {
+                    float4 sg = make_float4(0.f, 0.f, 0.f, 0.f), sb = sg;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int r = 8 * i + rs;
+                        const float rr = __shfl_sync(0xffffffffu, rstd, r);
+                        const float a1 = __shfl_sync(0xffffffffu, m1, r), a2 = __shfl_sync(0xffffffffu, m2, r);
+                        const float4 g = x[i], xh = u[i];
+                        if (r < nv) {   // clamped rows are not counted
+                            sg = make_float4(sg.x + g.x * xh.x, sg.y + g.y * xh.y, sg.z + g.z * xh.z, sg.w + g.w * xh.w);
+                            sb = add4(sb, g);
+                        }
+                        // g gamma as rounded for the sums: equal terms cancel exactly (one column: dz = 0)
+                        auto dz = [&](float gg, float gm, float h) { return rr * (__fmul_rn(gg, gm) - a1 - h * a2); };
+                        u[i] = make_float4(dz(g.x, ga.x, xh.x), dz(g.y, ga.y, xh.y), dz(g.z, ga.z, xh.z),
+                                           dz(g.w, ga.w, xh.w));
+                    }
+                    // column sums over the warp's rows
+                    float cs[8] = {sg.x, sg.y, sg.z, sg.w, sb.x, sb.y, sb.z, sb.w};
+#pragma unroll
+                    for (int o = 4; o < 32; o <<= 1) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) cs[i] += __shfl_xor_sync(0xffffffffu, cs[i], o);
+                    }
+                    if (lane < 4) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            sums[col + i] += cs[i];
+                            sums[NP + col + i] += cs[4 + i];
+                        }
+                    }
+                } else if constexpr (MODE == kEluAdjoint) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        u[i] = make_float4(u[i].x * elu1_deriv_from_out(x[i].x), u[i].y * elu1_deriv_from_out(x[i].y),
+                                           u[i].z * elu1_deriv_from_out(x[i].z), u[i].w * elu1_deriv_from_out(x[i].w));
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        u[i] = add4(u[i], b);
+                        if constexpr (OPS == kOpsRow) u[i] = add4(u[i], x[i]);
+                    }
+                }
+                // the next piece's operands (an in-place sum reads other columns than it has written)
+                if (MODE != kLnAdjoint && c0 + 16 < NP) load_ops(c0 + 16, x, y);
+                if constexpr (MODE == kElu) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 lo = elu_pair(make_float2(u[i].x, u[i].y)), hi = elu_pair(make_float2(u[i].z, u[i].w));
+                        u[i] = make_float4(lo.x, lo.y, hi.x, hi.y);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (8 * i + rs < nv) store4<VEC>(A.out + row[i] * A.ldo + col, nc, u[i]);
+                __syncwarp();
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty + eg);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if constexpr (MODE == kLnAdjoint) {
+        const float* z = reinterpret_cast<const float*>(sm + P.sums);
+        for (int i = tid; i < 2 * N; i += kThreads) {
+            const int o = (i < N) ? i : NP + (i - N);
+            float s = 0.f;
+            for (int w = 0; w < kEpilogueWarps; ++w) s += z[w * 2 * NP + o];
+            A.part[(int64_t)blockIdx.x * 2 * N + i] = s;
+        }
+    }
+    if (warp == 0) tmem_dealloc(tmem, NCOLS);
+}
+
+// ------------------------------------------------------------------ k_wgrad3
+
+struct WArgs {
+    int64_t rows;
+    int n_tiles;               // of RT rows
+    int RT;                    // rows per stage: 128, or 64 when an operand is 128 wide
+    const float* G;
+    const float* X;
+    int64_t ldg, ldx;
+    int N, K, NP, db, vec_g, vec_x, stages;
+    float* part;
+};
+
+struct WSmem {
+    uint32_t st, red, bar, tm, total, gterm, xterm, stage;
+};
+
+__host__ __device__ inline WSmem wgrad_smem(int NP, int KP, int RT, int stages) {
+    WSmem s;
+    s.gterm = (uint32_t)RT * NP * 2;
+    s.xterm = (uint32_t)RT * KP * 2;
+    s.stage = 3 * (s.gterm + s.xterm);
+    s.st = 0;
+    // M = 128 views of a narrower G read up to 256 RT bytes from a term's start: inside the
+    // stages, or in the pad behind the last one
+    uint32_t end = (uint32_t)stages * s.stage;
+    end = std::max(end, (uint32_t)(stages - 1) * s.stage + 2 * s.gterm + 256u * RT);
+    s.red = align_up(end, 16);                        // db: [128 threads][8]
+    s.bar = align_up(s.red + kSide * 8 * 4, 8);  // full[4], empty[4], acc_full[2], acc_empty[2]
+    s.tm = s.bar + 12 * 8;
+    s.total = s.tm + 16 + 1024;
+    return s;
+}
+
+struct WSide {
+    const float* src;
+    int64_t ld;
+    int cols;
+    uint32_t dst;   // of stage 0
+};
+
+// Load, split and write one operand's rows of every stage: [R x W], and their
+// column sums (cs: the thread's 8 columns, rows in order).
+template <int W, int R, bool VEC>
+__device__ __forceinline__ void wgrad_producer(const WArgs& A, const WSmem& P, const WSide& d, uint8_t* sm,
+                                               uint64_t* full, uint64_t* empty, int pt, int lane, float* cs) {
+    constexpr int U = W / 8, RS = kSide / U, IT = R / RS, B = IT < 4 ? IT : 4, S = span_of(W);
+    constexpr uint32_t TERM = R * W * 2;
+    const int c = (pt % U) * 8, row0 = pt / U, nc = d.cols - c;
+    const uint32_t off0 = tile_off(row0, c, R, S);
+    // rows RS apart: whole swizzle periods (1024 bytes) except the 128-wide rows, 8 apart, with the same period
+    static_assert((RS * S) % 1024 == 0, "the swizzle repeats every RS rows");
+    const int64_t step = RS * d.ld;
+    int st = 0, use = 0;
+    for (int t = blockIdx.x; t < A.n_tiles; t += gridDim.x) {
+        if (VEC && pt == 0 && d.ld == d.cols && t + (int)gridDim.x < A.n_tiles) {   // the next tile's rows into L2
+            const int64_t rn = (int64_t)(t + (int)gridDim.x) * R;
+            prefetch_l2(d.src + rn * d.ld, (uint32_t)(std::min<int64_t>(R, A.rows - rn) * d.cols * 4));
+        }
+        const int left = (int)std::min<int64_t>(R, A.rows - (int64_t)t * R);
+        const float* src = d.src + ((int64_t)t * R + row0) * d.ld + c;
+        uint8_t* dst = sm + d.dst + (uint32_t)st * P.stage + off0;
+#pragma unroll
+        for (int i0 = 0; i0 < IT; i0 += B) {
+            float v[B][8];
+            if (left == R && d.cols == W) {
+#pragma unroll
+                for (int i = 0; i < B; ++i) load8<VEC>(src + (i0 + i) * step, 8, v[i]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < B; ++i)
+                    load8<VEC>(src + (i0 + i) * step, row0 + (i0 + i) * RS < left ? nc : 0, v[i]);
+            }
+            if (i0 == 0 && use > 0 && !warp_wait(empty + st, (uint32_t)(use - 1) & 1u, lane)) return;
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) cs[k] += v[i][k];
+                uint4 h, m, l;
+                split8(v[i], h, m, l);
+                uint8_t* q = dst + (i0 + i) * RS * S;
+                *reinterpret_cast<uint4*>(q) = h;
+                *reinterpret_cast<uint4*>(q + TERM) = m;
+                *reinterpret_cast<uint4*>(q + 2 * TERM) = l;
+            }
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full + st);
+        if (++st == A.stages) {
+            st = 0;
+            ++use;
+        }
+    }
+}
+
+// dW = G^T X over the CTA's row tiles: both operands are MN-major views of the
+// same split row tiles (rows = the contraction). The accumulator of one tile
+// (RT rows) is added to FP32 registers by the epilogue warps, so no tensor-core
+// sum runs over more than RT rows.
+template <int KP>
+__global__ void __launch_bounds__(kWThreads, 1) k_wgrad3(const __grid_constant__ WArgs A) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* sm = aligned_smem(smem_raw);
+    const int NP = A.NP, RT = A.RT, stages = A.stages, N = A.N, K = A.K;
+    const int Sg = span_of(NP);
+    constexpr int Sx = span_of(KP);
+    const WSmem P = wgrad_smem(NP, KP, RT, stages);
+    uint64_t* full = reinterpret_cast<uint64_t*>(sm + P.bar);
+    uint64_t* empty = full + 4;
+    uint64_t* acc_full = full + 8;
+    uint64_t* acc_empty = full + 10;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + P.tm);
+    float* sRed = reinterpret_cast<float*>(sm + P.red);
+    constexpr uint32_t NCOLS = 2 * KP < 32 ? 32 : 2 * KP;
+    constexpr int CW = KP >= 32 ? KP / 2 : 16;      // accumulator columns per epilogue thread
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    if (warp == 0) {
+        tmem_alloc(tslot, NCOLS);
+        tmem_relinquish();
+    }
+    if (tid == 0) {
+        for (int i = 0; i < stages; ++i) {
+            mbar_init(full + i, kWProducerWarps);
+            mbar_init(empty + i, 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(acc_full + i, 1);
+            mbar_init(acc_empty + i, kEpilogueWarps);
+        }
+        fence_mbar_init();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot;
+    float* part = A.part + (int64_t)blockIdx.x * (N * K + (A.db ? N : 0));
+
+    if (warp < kWProducerWarps) {
+        // half of the producer warps split G, half X
+        const bool x = warp >= kWProducerWarps / 2;
+        const int pt = tid & (kSide - 1);
+        const WSide d{x ? A.X : A.G, x ? A.ldx : A.ldg, x ? K : N, P.st + (x ? 3 * P.gterm : 0u)};
+        float cs[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) cs[i] = 0.f;
+        auto go = [&](auto w, auto rt) {
+            constexpr int W = decltype(w)::value, R = decltype(rt)::value;
+            if (x ? A.vec_x : A.vec_g) wgrad_producer<W, R, true>(A, P, d, sm, full, empty, pt, lane, cs);
+            else wgrad_producer<W, R, false>(A, P, d, sm, full, empty, pt, lane, cs);
+        };
+        const int w = x ? KP : NP;
+        if (RT == 64) {
+            if (w == 128) go(Int<128>(), Int<64>());
+            else if (w == 64) go(Int<64>(), Int<64>());
+            else if (w == 32) go(Int<32>(), Int<64>());
+            else go(Int<16>(), Int<64>());
+        } else {
+            if (w == 64) go(Int<64>(), Int<128>());
+            else if (w == 32) go(Int<32>(), Int<128>());
+            else go(Int<16>(), Int<128>());
+        }
+        if (A.db && !x) {   // column sums of G: threads of one column group in thread order
+            const int gu = NP / 8;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sRed[pt * 8 + k] = cs[k];
+            named_sync(1, kSide);
+            for (int c = pt; c < N; c += kSide) {
+                float s = 0.f;
+                for (int i = c / 8; i < kSide; i += gu) s += sRed[i * 8 + (c & 7)];
+                part[(int64_t)N * K + c] = s;
+            }
+        }
+    } else if (warp == kWProducerWarps + kEpilogueWarps) {
+        if (lane == 0) {
+            const uint32_t id = idesc_bf16(128, KP, 1, 1);
+            const uint32_t base = smem_u32(sm + P.st);
+            const uint64_t g0 = sdesc(base, (uint32_t)RT * Sg, 8 * Sg, swz_code(Sg));
+            const uint64_t x0 = sdesc(base + 3 * P.gterm, (uint32_t)RT * Sx, 8 * Sx, swz_code(Sx));
+            int n = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++n) {
+                const int st = n % stages, use = n / stages, buf = n & 1;
+                if (n >= 2) ok = mbar_wait(acc_empty + buf, (uint32_t)((n >> 1) - 1) & 1u);
+                ok = ok && mbar_wait(full + st, (uint32_t)use & 1u);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t d = tmem + (uint32_t)(buf * KP), so = (uint32_t)st * P.stage;
+                auto issue = [&](auto rt) {
+#pragma unroll
+                    for (int p = 0; p < 6; ++p) {
+                        const uint64_t gp = desc_step(g0, so + kTermA[p] * P.gterm);
+                        const uint64_t xp = desc_step(x0, so + kTermB[p] * P.xterm);
+#pragma unroll
+                        for (int k0 = 0; k0 < decltype(rt)::value; k0 += 16)
+                            mma_bf16(d, desc_step(gp, (uint32_t)(k0 * Sg)), desc_step(xp, (uint32_t)(k0 * Sx)), id,
+                                     (p > 0 || k0 > 0) ? 1u : 0u);
+                    }
+                };
+                if (RT == 64) issue(Int<64>());
+                else issue(Int<128>());
+                mma_commit(empty + st);
+                mma_commit(acc_full + buf);
+            }
+            if (ok && n > 0) mbar_wait(empty + (n - 1) % stages, (uint32_t)((n - 1) / stages) & 1u);
+        }
+        __syncwarp();
+    } else {
+        const int ew = warp - kWProducerWarps, q = ew & 3, half = ew >> 2;
+        const int c0 = half * CW;
+        const bool work = c0 < KP;
+        float acc[CW];
+#pragma unroll
+        for (int i = 0; i < CW; ++i) acc[i] = 0.f;
+        int n = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++n) {
+            const int buf = n & 1;
+            ok = warp_wait(acc_full + buf, (uint32_t)(n >> 1) & 1u, lane);
+            if (!ok) break;
+            tc_fence_after();
+            if (work) {
+#pragma unroll
+                for (int i = 0; i < CW; i += 16) {
+                    float v[16];
+                    tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * KP + c0 + i), v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) acc[i + k] += v[k];
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty + buf);
+        }
+        const int r = 32 * q + lane;
+        if (work && r < N) {
+#pragma unroll
+            for (int i = 0; i < CW; ++i)
+                if (c0 + i < K) part[(int64_t)r * K + c0 + i] = acc[i];
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0) tmem_dealloc(tmem, NCOLS);
+}
+
+// ------------------------------------------------------------------ k_reduce3
+
+struct RedArgs {
+    Sum s[kMaxReduce];
+    int first[kMaxReduce + 1];   // first block of each sum
+    int n;
+};
+
+// 32 elements x 8 lanes over the partials of a block: lane l sums the partials
+// l, l + 8, ... in order, and the lanes are combined in order.
+__global__ void __launch_bounds__(256) k_reduce3(const __grid_constant__ RedArgs A) {
+    __shared__ float red[8][33];
+    int i = 0;
+    while (i + 1 < A.n && (int)blockIdx.x >= A.first[i + 1]) ++i;
+    const Sum& S = A.s[i];
+    const int cx = threadIdx.x & 31, l = threadIdx.x >> 5;
+    const int e = ((int)blockIdx.x - A.first[i]) * 32 + cx;
+    float s = 0.f;
+    if (e < S.N * S.K) {
+        const float* p = S.part + e;
+#pragma unroll 4
+        for (int z = l; z < S.nz; z += 8) s += p[(int64_t)z * S.stride];
+    }
+    red[l][cx] = s;
+    __syncthreads();
+    if (l == 0 && e < S.N * S.K) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t += red[k][cx];
+        float* d = S.dst + (int64_t)(e / S.K) * S.ldd + e % S.K;
+        *d += t;
+    }
+}
+
+inline bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
+
+template <class Kern>
+int set_smem(Kern k, uint32_t bytes) {
+    GNN_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
+                   "cudaFuncSetAttribute");
+    return GNN_OK;
+}
+
+int pick_stages(int NP, int KB, int nkb) {
+    for (int s = 4; s >= 2; --s)
+        if (lin_smem(NP, KB, nkb, s).total <= kSmemMax) return s;
+    return 0;
+}
+
+int blocks_of(int K, int KB) { return K ? (pow2_width(K) + KB - 1) / KB : 0; }
+int block_width(int K) { return std::min(64, pow2_width(K)); }
+
+}  // namespace
+
+bool fits(int N, int K, int sources) {
+    if (N > kMaxWidth || K > kMaxWidth) return false;
+    const int KB = block_width(K);
+    return pick_stages(pad16(N), KB, sources * blocks_of(K, KB)) != 0;
+}
+
+int run(Mode mode, Args a, cudaStream_t s, int* ctas) {
+    if (ctas) *ctas = 0;
+    if (a.rows == 0 || a.N == 0) return GNN_OK;
+    const int64_t nt = (a.rows + 127) / 128;
+    GNN_REQUIRE(nt <= 0x7fffffff - 2 * kMaxCtas, GNN_ESHAPE, "lin3: too many rows");
+    a.n_tiles = (int)nt;
+    a.NP = pad16(a.N);
+    a.KB = block_width(std::max(a.K[0], a.K[1]));
+    a.nkb[0] = blocks_of(a.K[0], a.KB);
+    a.nkb[1] = blocks_of(a.K[1], a.KB);
+    a.stages = pick_stages(a.NP, a.KB, a.nkb[0] + a.nkb[1]);
+    GNN_REQUIRE(a.stages > 0 && a.N <= kMaxWidth, GNN_EUNSUPPORTED, "lin3: shape %d x (%d + %d) does not fit", a.N,
+                a.K[0], a.K[1]);
+    // 16-byte accesses only where every row of every operand starts on a 16-byte boundary
+    bool vec = a.N % 4 == 0 && aligned16(a.out) && a.ldo % 4 == 0;
+    for (int i = 0; i < 2; ++i)
+        if (a.K[i]) vec = vec && a.K[i] % 4 == 0 && a.lda[i] % 4 == 0 && aligned16(a.A[i]);
+    vec = vec && (!a.add || (aligned16(a.add) && a.ldadd % 4 == 0));
+    vec = vec && (!a.P || (aligned16(a.P) && aligned16(a.Q) && a.ldpq % 4 == 0));
+    vec = vec && aligned16(a.g0) && aligned16(a.da) && aligned16(a.g_out);
+    if (a.nsplit <= 0) a.nsplit = a.NP;
+    const uint32_t smem = lin_smem(a.NP, a.KB, a.nkb[0] + a.nkb[1], a.stages).total;
+    const int grid = (int)std::min<int64_t>(nt, std::min(kMaxCtas, fused::host::num_sms()));
+    if (ctas) *ctas = grid;
+    int rc = GNN_OK;
+    auto launch = [&](auto mode_c, auto ops_c, const char* name) {
+        constexpr int M = decltype(mode_c)::value, O = decltype(ops_c)::value;
+        auto kern = vec ? k_lin3<M, O, true> : k_lin3<M, O, false>;
+        if ((rc = set_smem(kern, smem))) return;
+        ProfScope _ps(s, name);
+        kern<<<grid, kThreads, smem, s>>>(a);
+    };
+    constexpr Int<kOpsNone> none;
+    constexpr Int<kOpsRow> one_row;
+    constexpr Int<kOpsGather> gather;
+    switch (mode) {
+        case kElu:
+            if (a.P) launch(Int<kElu>(), gather, "k_lin3_elu");
+            else if (a.add) launch(Int<kElu>(), one_row, "k_lin3_elu");
+            else launch(Int<kElu>(), none, "k_lin3_elu");
+            break;
+        case kLayerNorm:
+            if (a.add) launch(Int<kLayerNorm>(), one_row, "k_lin3_ln");
+            else launch(Int<kLayerNorm>(), none, "k_lin3_ln");
+            break;
+        case kLnAdjoint:
+            if (a.da) launch(Int<kLnAdjoint>(), gather, "k_lin3_ln_adj");
+            else launch(Int<kLnAdjoint>(), none, "k_lin3_ln_adj");
+            break;
+        case kEluAdjoint: launch(Int<kEluAdjoint>(), one_row, "k_lin3_elu_adj"); break;
+        case kAdd:
+            if (a.add) launch(Int<kAdd>(), one_row, "k_lin3_add");
+            else launch(Int<kAdd>(), none, "k_lin3_add");
+            break;
+    }
+    if (rc) return rc;
+    GNN_LAUNCH_CHECK("k_lin3");
+    return GNN_OK;
+}
+
+int wgrad(int64_t rows, const float* G, int64_t ldg, int N, const float* X, int64_t ldx, int K, bool db, float* part,
+          cudaStream_t s, int* ctas) {
+    *ctas = 0;
+    if (rows == 0) return GNN_OK;
+    GNN_REQUIRE(N <= kMaxWidth && K <= kMaxWidth, GNN_EUNSUPPORTED, "lin3: weight gradient %d x %d does not fit", N, K);
+    WArgs a{};
+    a.rows = rows;
+    a.G = G; a.ldg = ldg; a.N = N;
+    a.X = X; a.ldx = ldx; a.K = K;
+    a.NP = pow2_width(N);
+    const int KP = pow2_width(K);
+    a.RT = (a.NP > 64 || KP > 64) ? 64 : 128;
+    const int64_t nt = (rows + a.RT - 1) / a.RT;
+    GNN_REQUIRE(nt <= 0x7fffffff - 2 * kMaxCtas, GNN_ESHAPE, "lin3: too many rows");
+    a.n_tiles = (int)nt;
+    a.db = db ? 1 : 0;
+    a.vec_g = N % 4 == 0 && ldg % 4 == 0 && aligned16(G);
+    a.vec_x = K % 4 == 0 && ldx % 4 == 0 && aligned16(X);
+    a.stages = 4;
+    while (wgrad_smem(a.NP, KP, a.RT, a.stages).total > kSmemMax) --a.stages;
+    a.part = part;
+    const uint32_t smem = wgrad_smem(a.NP, KP, a.RT, a.stages).total;
+    const int grid = (int)std::min<int64_t>(nt, std::min(kMaxCtas, fused::host::num_sms()));
+    *ctas = grid;
+    int rc = GNN_OK;
+    auto launch = [&](auto kern) {
+        if ((rc = set_smem(kern, smem))) return;
+        ProfScope _ps(s, "k_wgrad3");
+        kern<<<grid, kWThreads, smem, s>>>(a);
+    };
+    if (KP == 16) launch(k_wgrad3<16>);
+    else if (KP == 32) launch(k_wgrad3<32>);
+    else if (KP == 64) launch(k_wgrad3<64>);
+    else launch(k_wgrad3<128>);
+    if (rc) return rc;
+    GNN_LAUNCH_CHECK("k_wgrad3");
+    return GNN_OK;
+}
+
+int reduce(const Sum* sums, int n, cudaStream_t s) {
+    RedArgs a{};
+    int blocks = 0;
+    for (int i = 0; i < n; ++i) {
+        if (sums[i].nz == 0 || !sums[i].dst) continue;
+        GNN_REQUIRE(a.n < kMaxReduce, GNN_EUNSUPPORTED, "lin3: too many sums");
+        a.s[a.n] = sums[i];
+        a.first[a.n++] = blocks;
+        blocks += (sums[i].N * sums[i].K + 31) / 32;
+    }
+    a.first[a.n] = blocks;
+    if (blocks == 0) return GNN_OK;
+    {
+        ProfScope _ps(s, "k_reduce3");
+        k_reduce3<<<blocks, 256, 0, s>>>(a);
+    }
+    GNN_LAUNCH_CHECK("k_reduce3");
+    return GNN_OK;
+}
+
+}  // namespace lin3
+}  // namespace gnn

@@ -1,17 +1,21 @@
-// Plain FP32 path of libgnnmp: unfused SIMT kernels, no tensor cores, no TF32.
+// FP32 path of libgnnmp: FP32 states, weights, sums and results throughout.
 //
-// This is the straightforward reading of the consistent NMP layer (Eq. 5a-5e)
-// and its adjoint, one kernel per operation with every intermediate in
-// workspace memory. It is the FP32 correctness and speed baseline the fused
-// BF16 path is measured against. All reductions run in a fixed order:
-// CSR segmented sums over receiver (or sender) lists, split-K partial products
-// reduced in chunk order, and block-partial column sums reduced in block
-// order, so two runs give bitwise equal results.
+// MLPs whose widths are at most 128 run one tensor-core kernel per Linear
+// (lin3.cu: FP32 operands as exact sums of three BF16 numbers), with bias,
+// ELU, LayerNorm, residual, gathers and their adjoints in its epilogue; the
+// edge MLP's first Linear is split into two products per node and one per
+// edge, W1 [x_i, x_j, e] = P_i + Q_j + W1c e. Wider MLPs run the unfused SIMT
+// kernels below, one per operation, with every intermediate in workspace
+// memory. All reductions run in a fixed order: CSR segmented sums over
+// receiver (or sender) lists, partial products reduced in chunk order, and
+// block-partial column sums reduced in block order, so two runs give bitwise
+// equal results.
 
 #include <algorithm>
 #include <cstring>
 
 #include "device_common.cuh"
+#include "lin3.h"
 #include "plain.h"
 #include "profiler.h"
 
@@ -363,6 +367,78 @@ __global__ void k_edge_grad_out(const float* __restrict__ de_tot, const float* _
     de_in[i] = de_tot[i] + dX1[e * 3 * H + 2 * H + c];
 }
 
+// recv[e] = receiver row of edge e.
+__global__ void k_receivers(const int32_t* __restrict__ row_ptr, int64_t rows, int32_t* __restrict__ recv) {
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= rows) return;
+    for (int32_t e = row_ptr[r]; e < row_ptr[r + 1]; ++e) recv[e] = (int32_t)r;
+}
+
+// Sums of a node's edge rows, V columns per thread (V = 4 when rows start on
+// 16-byte boundaries): the terms in edge order, four loads in flight.
+template <int V>
+struct RowVec;
+template <>
+struct RowVec<1> {
+    float v;
+    __device__ void zero() { v = 0.f; }
+    __device__ static RowVec load(const float* p) { return {__ldg(p)}; }
+    __device__ void fma(float w, const RowVec& o) { v = fmaf(w, o.v, v); }
+    __device__ void add(const RowVec& o) { v += o.v; }
+    __device__ void store(float* p) const { *p = v; }
+};
+template <>
+struct RowVec<4> {
+    float4 v;
+    __device__ void zero() { v = make_float4(0.f, 0.f, 0.f, 0.f); }
+    __device__ static RowVec load(const float* p) { return {__ldg(reinterpret_cast<const float4*>(p))}; }
+    __device__ void fma(float w, const RowVec& o) {
+        v = make_float4(fmaf(w, o.v.x, v.x), fmaf(w, o.v.y, v.y), fmaf(w, o.v.z, v.z), fmaf(w, o.v.w, v.w));
+    }
+    __device__ void add(const RowVec& o) { v = make_float4(v.x + o.v.x, v.y + o.v.y, v.z + o.v.z, v.w + o.v.w); }
+    __device__ void store(float* p) const { *reinterpret_cast<float4*>(p) = v; }
+};
+
+// a[r] = sum over edges e of r (ascending) of w[e] * Y[e]              (Eq. 5b)
+template <int V>
+__global__ void k_segsum_rows(const int32_t* __restrict__ row_ptr, const float* __restrict__ w, int64_t rows, int H,
+                              const float* __restrict__ Y, float* __restrict__ a) {
+    const int per = H / V;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= rows * per) return;
+    const int64_t r = i / per;
+    const int c = (int)(i - r * per) * V;
+    RowVec<V> s;
+    s.zero();
+    const int32_t e1 = row_ptr[r + 1];
+#pragma unroll 4
+    for (int32_t e = row_ptr[r]; e < e1; ++e) s.fma(__ldg(w + e), RowVec<V>::load(Y + (int64_t)e * H + c));
+    s.store(a + r * H + c);
+}
+
+// dP[r] = sum of dz over the edges received by r, dQ[r] = over those sent by r
+// (adjoints of the per-node products of the first edge Linear).
+template <int V>
+__global__ void k_node_sums(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ t_ptr,
+                            const int32_t* __restrict__ t_eid, int64_t rows, int H, const float* __restrict__ dz,
+                            float* __restrict__ dP, float* __restrict__ dQ) {
+    const int per = H / V;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= rows * per) return;
+    const int64_t r = i / per;
+    const int c = (int)(i - r * per) * V;
+    RowVec<V> s, t;
+    s.zero();
+    t.zero();
+    const int32_t e1 = row_ptr[r + 1], k1 = t_ptr[r + 1];
+#pragma unroll 4
+    for (int32_t e = row_ptr[r]; e < e1; ++e) s.add(RowVec<V>::load(dz + (int64_t)e * H + c));
+#pragma unroll 4
+    for (int32_t k = t_ptr[r]; k < k1; ++k) t.add(RowVec<V>::load(dz + (int64_t)__ldg(t_eid + k) * H + c));
+    s.store(dP + r * H + c);
+    t.store(dQ + r * H + c);
+}
+
 // Eq. 5c-5d on one device: each shared id's copies are summed in list order
 // (increasing sub-graph) and the sum written back to every copy.
 __global__ void k_halo(const int32_t* __restrict__ halo_ptr, const int32_t* __restrict__ halo_rows,
@@ -659,7 +735,317 @@ struct Carve {
     }
 };
 
-// ------------------------------------------------------------------ MP layer, plain FP32
+
+// ------------------------------------------------------------------ MLPs on the tensor cores (lin3)
+
+// The tensor-core Linears cover MLPs of widths up to 128 (the first layer's
+// concatenated inputs counted per source). They are faster over the whole
+// range they cover; wider MLPs need more shared memory than a block has.
+static bool tc_widths(const gnn_mlp& P, int in) {
+    if (in > lin3::kMaxWidth) return false;
+    for (int k = 1; k <= P.n_lin; ++k)
+        if (P.dims[k] > lin3::kMaxWidth) return false;
+    return true;
+}
+static bool tc_layer(const gnn_mp_config& cfg) { return cfg.hidden <= lin3::kMaxWidth; }
+
+static bool vec4(int H, const void* a, const void* b, const void* c) {
+    return H % 4 == 0 && (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c) & 15) == 0;
+}
+
+// out = op(X W^T + b): one source X [rows x K], W [N x K]
+static lin3::Args lin_args(int64_t rows, const float* X, int64_t ldx, int K, const float* W, int64_t ldw, int N,
+                           const float* bias, float* out, int64_t ldo) {
+    lin3::Args a{};
+    a.rows = rows;
+    a.A[0] = X; a.lda[0] = ldx; a.K[0] = K;
+    a.W[0] = W; a.sn = ldw; a.sk = 1;
+    a.N = N; a.bias = bias; a.out = out; a.ldo = ldo;
+    return a;
+}
+// out = op(G W): G [rows x N], W [N x K] (its columns k0 .. k0 + K of ldw)
+static lin3::Args dgrad_args(int64_t rows, const float* G, int N, const float* W, int64_t ldw, int K, float* out,
+                             int64_t ldo) {
+    lin3::Args a{};
+    a.rows = rows;
+    a.A[0] = G; a.lda[0] = N; a.K[0] = N;
+    a.W[0] = W; a.sn = 1; a.sk = ldw;
+    a.N = K; a.out = out; a.ldo = ldo;
+    return a;
+}
+
+// The hidden Linears 1 .. n_lin-2 from hbuf[1] (hbuf[k] = input of Linear k).
+static int tc_hidden(const gnn_mlp& P, int64_t rows, float* const* hbuf, cudaStream_t s) {
+    for (int k = 1; k + 1 < P.n_lin; ++k) {
+        lin3::Args a = lin_args(rows, hbuf[k], P.dims[k], P.dims[k], P.W[k], P.dims[k], P.dims[k + 1], P.b[k],
+                                hbuf[k + 1], P.dims[k + 1]);
+        int rc = lin3::run(lin3::kElu, a, s);
+        if (rc) return rc;
+    }
+    return GNN_OK;
+}
+
+// Last Linear with LayerNorm and residual (res may be NULL), or plain without LayerNorm.
+static int tc_last(const gnn_mlp& P, int64_t rows, float* const* hbuf, float eps, const float* res, float* out,
+                   cudaStream_t s) {
+    const int k = P.n_lin - 1;
+    lin3::Args a = lin_args(rows, hbuf[k], P.dims[k], P.dims[k], P.W[k], P.dims[k], P.dims[k + 1], P.b[k], out,
+                            P.dims[k + 1]);
+    a.add = res; a.ldadd = P.dims[k + 1];
+    a.gamma = P.gamma; a.beta = P.beta; a.eps = eps;
+    return lin3::run(P.gamma ? lin3::kLayerNorm : lin3::kAdd, a, s);
+}
+
+// Sums of a backward pass, reduced into the gradients by one launch at its end.
+struct GradSums {
+    lin3::Sum s[lin3::kMaxReduce];
+    int n = 0;
+    float* part;   // next free partials
+    explicit GradSums(float* p) : part(p) {}
+    int flush(cudaStream_t st) {
+        int rc = lin3::reduce(s, n, st);
+        n = 0;
+        return rc;
+    }
+    // dW [N x K] (row stride ldw) += G^T X, db += column sums of G (db may be NULL)
+    int weight(int64_t rows, const float* G, int N, const float* X, int64_t ldx, int K, float* dW, int64_t ldw,
+               float* db, cudaStream_t st) {
+        int nz = 0;
+        int rc = lin3::wgrad(rows, G, N, N, X, ldx, K, db != nullptr, part, st, &nz);
+        if (rc) return rc;
+        const int64_t stride = (int64_t)N * K + (db ? N : 0);
+        s[n++] = {part, stride, nz, N, K, dW, ldw};
+        if (db) s[n++] = {part + (int64_t)N * K, stride, nz, 1, N, db, N};
+        part += lin3::wgrad_floats(N, K);
+        return GNN_OK;
+    }
+};
+static int64_t tc_grad_floats(const gnn_mlp& P, int in, int sources) {
+    int64_t f = (int64_t)lin3::kMaxCtas * 2 * P.dims[P.n_lin] + sources * lin3::wgrad_floats(P.dims[1], in);
+    for (int k = 1; k < P.n_lin; ++k) f += lin3::wgrad_floats(P.dims[k + 1], P.dims[k]);
+    return f;
+}
+
+// Adjoint of the last Linear's LayerNorm and of Linears n_lin-1 .. 1, from the
+// recomputed inputs hbuf[k]: returns dL/d(pre-activation 0) in *dz0 (one of
+// g0, g1). a: the upstream gradient's arguments (g0, da, w, recv, g_out);
+// without LayerNorm the upstream gradient is dY itself.
+static int tc_chain_bwd(const gnn_mlp& P, const gnn_mlp& dP, int64_t rows, float* const* hbuf, float eps,
+                        const lin3::Args& up, const float* dY, float* g0, float* g1, const float** dz0, GradSums& gs,
+                        cudaStream_t s) {
+    const int n = P.n_lin, H = P.dims[n];
+    const float* g = dY;
+    int rc;
+    if (P.gamma) {
+        lin3::Args a = lin_args(rows, hbuf[n - 1], P.dims[n - 1], P.dims[n - 1], P.W[n - 1], P.dims[n - 1], H,
+                                P.b[n - 1], g0, H);
+        a.gamma = P.gamma; a.beta = P.beta; a.eps = eps;
+        a.g0 = up.g0; a.da = up.da; a.w = up.w; a.recv = up.recv; a.g_out = up.g_out;
+        a.part = gs.part;
+        int nz = 0;
+        if ((rc = lin3::run(lin3::kLnAdjoint, a, s, &nz))) return rc;
+        gs.s[gs.n++] = {gs.part, 2 * H, nz, 1, H, dP.gamma, H};
+        gs.s[gs.n++] = {gs.part + H, 2 * H, nz, 1, H, dP.beta, H};
+        gs.part += (int64_t)lin3::kMaxCtas * 2 * H;
+        g = g0;
+    }
+    float* next = g == g0 ? g1 : g0;
+    for (int k = n - 1; k >= 1; --k) {
+        const int N = P.dims[k + 1], K = P.dims[k];
+        if ((rc = gs.weight(rows, g, N, hbuf[k], K, K, dP.W[k], K, dP.b[k], s))) return rc;
+        lin3::Args a = dgrad_args(rows, g, N, P.W[k], K, K, next, K);
+        a.add = hbuf[k]; a.ldadd = K;
+        if ((rc = lin3::run(lin3::kEluAdjoint, a, s))) return rc;
+        g = next;
+        next = g == g0 ? g1 : g0;
+    }
+    *dz0 = g;
+    return GNN_OK;
+}
+
+// ------------------------------------------------------------------ MP layer on the tensor cores
+
+struct TcBufs {
+    float* PQ;                    // [NR x 2H]: x W1a^T | x W1b^T
+    int32_t* recv;                // [E]
+    float* hE[GNN_MAX_LIN];
+    float* hN[GNN_MAX_LIN];
+    float* e_new;
+    float* a;
+    float *g0, *g1;               // backward: gradients of an MLP's running layer
+    float *da, *dP, *dQ;
+    float* part;
+};
+
+// keep: every MLP activation (the backward's recomputation); otherwise two buffers.
+static void carve_tc(Carve& c, const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_params& W, bool bwd,
+                     TcBufs& b) {
+    const int64_t NR = G.n_rows, E = G.n_edges, H = cfg.hidden, m = std::max(NR, E);
+    b = TcBufs{};
+    b.PQ = c.take<float>(NR * 2 * H);
+    b.recv = c.take<int32_t>(E);
+    b.a = c.take<float>(NR * H);
+    if (!bwd) {
+        float* pp[2] = {c.take<float>(m * H), c.take<float>(m * H)};
+        for (int k = 1; k < GNN_MAX_LIN; ++k) b.hE[k] = b.hN[k] = pp[k & 1];
+        b.e_new = c.take<float>(E * H);
+        return;
+    }
+    for (int k = 1; k < W.edge.n_lin; ++k) b.hE[k] = c.take<float>(E * H);
+    for (int k = 1; k < W.node.n_lin; ++k) b.hN[k] = c.take<float>(NR * H);
+    b.g0 = c.take<float>(m * H);
+    b.g1 = c.take<float>(m * H);
+    b.e_new = b.g0;               // only while a* is recomputed
+    b.da = c.take<float>(NR * H);
+    b.dP = c.take<float>(NR * H);
+    b.dQ = c.take<float>(NR * H);
+    b.part = c.take<float>(tc_grad_floats(W.edge, cfg.hidden, 3) + tc_grad_floats(W.node, cfg.hidden, 2));
+}
+
+// Receivers, P|Q and the edge MLP up to the input of its last Linear.
+static int tc_edge_hidden(const gnn_graph_dev& G, int H, const gnn_mlp& P, const float* x, const float* e, TcBufs& b,
+                          cudaStream_t s) {
+    const int64_t NR = G.n_rows, E = G.n_edges;
+    if (!NR || !E) return GNN_OK;
+    {
+        ProfScope _ps(s, "k_receivers");
+        k_receivers<<<grid1(NR), 256, 0, s>>>(G.row_ptr, NR, b.recv);
+    }
+    GNN_LAUNCH_CHECK("k_receivers");
+    int rc;
+    const bool one = lin3::fits(2 * H, H, 1);   // [W1a; W1b] as one [2H x H] weight
+    for (int h = 0; h < (one ? 1 : 2); ++h) {
+        lin3::Args a = lin_args(NR, x, H, H, P.W[0] + h * H, 3 * H, one ? 2 * H : H, nullptr, b.PQ + h * H, 2 * H);
+        a.nsplit = H;
+        a.noff = H;
+        if ((rc = lin3::run(lin3::kAdd, a, s))) return rc;
+    }
+    lin3::Args a = lin_args(E, e, H, H, P.W[0] + 2 * H, 3 * H, H, P.b[0], b.hE[1], H);
+    a.P = b.PQ; a.Q = b.PQ + H; a.ldpq = 2 * H; a.recv = b.recv; a.snd = G.col;
+    if ((rc = lin3::run(lin3::kElu, a, s))) return rc;
+    return tc_hidden(P, E, b.hE, s);
+}
+
+// Edge update output, aggregation and halo sum (Eq. 5a-5d).
+static int tc_aggregate(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mlp& P, const float* e,
+                        float* e_new, float* a, TcBufs& b, cudaStream_t s) {
+    const int H = cfg.hidden;
+    const int64_t NR = G.n_rows;
+    int rc;
+    if ((rc = tc_last(P, G.n_edges, b.hE, cfg.ln_eps, e, e_new, s))) return rc;
+    if (NR) {
+        {
+            ProfScope _ps(s, "k_segsum");
+            if (vec4(H, e_new, a, nullptr))
+                k_segsum_rows<4><<<grid1(NR * (H / 4)), 256, 0, s>>>(G.row_ptr, G.edge_w, NR, H, e_new, a);
+            else
+                k_segsum_rows<1><<<grid1(NR * H), 256, 0, s>>>(G.row_ptr, G.edge_w, NR, H, e_new, a);
+        }
+        GNN_LAUNCH_CHECK("k_segsum");
+    }
+    return cfg.halo_mode == GNN_HALO_SYNC ? halo(G, a, H, s) : GNN_OK;
+}
+
+// The node MLP on [a, x] up to the input of its last Linear.
+static int tc_node_hidden(int64_t NR, int H, const gnn_mlp& P, const float* a_star, const float* x, TcBufs& b,
+                          cudaStream_t s) {
+    int rc;
+    if (lin3::fits(H, H, 2)) {
+        lin3::Args a = lin_args(NR, a_star, H, H, P.W[0], 2 * H, H, P.b[0], b.hN[1], H);
+        a.A[1] = x; a.lda[1] = H; a.K[1] = H; a.W[1] = P.W[0] + H;
+        if ((rc = lin3::run(lin3::kElu, a, s))) return rc;
+    } else {   // the two halves of the weight one after the other
+        lin3::Args a = lin_args(NR, a_star, H, H, P.W[0], 2 * H, H, nullptr, b.hN[1], H);
+        if ((rc = lin3::run(lin3::kAdd, a, s))) return rc;
+        a = lin_args(NR, x, H, H, P.W[0] + H, 2 * H, H, P.b[0], b.hN[1], H);
+        a.add = b.hN[1]; a.ldadd = H;
+        if ((rc = lin3::run(lin3::kElu, a, s))) return rc;
+    }
+    return tc_hidden(P, NR, b.hN, s);
+}
+
+static int tc_mp_forward(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_params& W, const float* x_in,
+                         const float* e_in, float* x_out, float* e_out, float* a_star_out, void* ws, cudaStream_t s) {
+    Carve c(ws);
+    TcBufs b;
+    carve_tc(c, G, cfg, W, false, b);
+    float* a = a_star_out ? a_star_out : b.a;
+    int rc;
+    if ((rc = tc_edge_hidden(G, cfg.hidden, W.edge, x_in, e_in, b, s))) return rc;
+    if ((rc = tc_aggregate(G, cfg, W.edge, e_in, e_out ? e_out : b.e_new, a, b, s))) return rc;
+    if ((rc = tc_node_hidden(G.n_rows, cfg.hidden, W.node, a, x_in, b, s))) return rc;
+    return tc_last(W.node, G.n_rows, b.hN, cfg.ln_eps, x_in, x_out, s);   // Eq. 5e
+}
+
+static int tc_mp_backward(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_params& W, const float* x_in,
+                          const float* e_in, const float* a_star, const float* dx_out, const float* de_out,
+                          float* dx_in, float* de_in, const gnn_mp_params& dW, void* ws, cudaStream_t s) {
+    const int H = cfg.hidden;
+    const int64_t NR = G.n_rows, E = G.n_edges;
+    Carve c(ws);
+    TcBufs b;
+    carve_tc(c, G, cfg, W, true, b);
+    int rc;
+    // recompute the activations of this layer
+    if ((rc = tc_edge_hidden(G, H, W.edge, x_in, e_in, b, s))) return rc;
+    const float* a = a_star;
+    if (!a) {
+        if ((rc = tc_aggregate(G, cfg, W.edge, e_in, b.e_new, b.a, b, s))) return rc;
+        a = b.a;
+    }
+    if ((rc = tc_node_hidden(NR, H, W.node, a, x_in, b, s))) return rc;
+
+    // node update adjoint (Eq. 5e)
+    GradSums gs(b.part);
+    const float* dz = nullptr;
+    lin3::Args up{};
+    up.g0 = dx_out;
+    if ((rc = tc_chain_bwd(W.node, dW.node, NR, b.hN, cfg.ln_eps, up, nullptr, b.g0, b.g1, &dz, gs, s))) return rc;
+    if ((rc = gs.weight(NR, dz, H, a, H, H, dW.node.W[0], 2 * H, dW.node.b[0], s))) return rc;
+    if ((rc = gs.weight(NR, dz, H, x_in, H, H, dW.node.W[0] + H, 2 * H, nullptr, s))) return rc;
+    lin3::Args l = dgrad_args(NR, dz, H, W.node.W[0], 2 * H, H, b.da, H);
+    if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
+    l = dgrad_args(NR, dz, H, W.node.W[0] + H, 2 * H, H, dx_in, H);
+    l.add = dx_out; l.ldadd = H;
+    if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
+    if ((rc = gs.flush(s))) return rc;
+    // halo swap + sync adjoint (Eq. 5c-5d): the same symmetric copy-sum
+    if (cfg.halo_mode == GNN_HALO_SYNC && (rc = halo(G, b.da, H, s))) return rc;
+
+    // edge update adjoint (Eq. 5a): the gradient of e' is de_out + w da_i (adjoint of Eq. 5b), kept in de_in
+    up = lin3::Args{};
+    up.g0 = de_out; up.da = b.da; up.w = G.edge_w; up.recv = b.recv; up.g_out = de_in;
+    if ((rc = tc_chain_bwd(W.edge, dW.edge, E, b.hE, cfg.ln_eps, up, nullptr, b.g0, b.g1, &dz, gs, s))) return rc;
+    if (E && (rc = gs.weight(E, dz, H, e_in, H, H, dW.edge.W[0] + 2 * H, 3 * H, dW.edge.b[0], s))) return rc;
+    if (NR) {
+        {
+            ProfScope _ps(s, "k_node_sums");
+            if (vec4(H, dz, b.dP, b.dQ))
+                k_node_sums<4><<<grid1(NR * (H / 4)), 256, 0, s>>>(G.row_ptr, G.t_ptr, G.t_eid, NR, H, dz, b.dP, b.dQ);
+            else
+                k_node_sums<1><<<grid1(NR * H), 256, 0, s>>>(G.row_ptr, G.t_ptr, G.t_eid, NR, H, dz, b.dP, b.dQ);
+        }
+        GNN_LAUNCH_CHECK("k_node_sums");
+    }
+    l = dgrad_args(E, dz, H, W.edge.W[0] + 2 * H, 3 * H, H, de_in, H);
+    l.add = de_in; l.ldadd = H;
+    if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
+    if ((rc = gs.weight(NR, b.dP, H, x_in, H, H, dW.edge.W[0], 3 * H, nullptr, s))) return rc;
+    if ((rc = gs.weight(NR, b.dQ, H, x_in, H, H, dW.edge.W[0] + H, 3 * H, nullptr, s))) return rc;
+    l = dgrad_args(NR, b.dP, H, W.edge.W[0], 3 * H, H, dx_in, H);
+    l.add = dx_in; l.ldadd = H;
+    if (lin3::fits(H, H, 2)) {
+        l.A[1] = b.dQ; l.lda[1] = H; l.K[1] = H; l.W[1] = W.edge.W[0] + H;
+        if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
+    } else {
+        if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
+        l.A[0] = b.dQ; l.W[0] = W.edge.W[0] + H;
+        if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
+    }
+    return gs.flush(s);
+}
+
+// ------------------------------------------------------------------ MP layer, SIMT (H > 128)
 
 struct LayerFwdBufs {
     float* X1;
@@ -738,6 +1124,11 @@ static int layer_forward_core(const gnn_graph_dev& G, const gnn_mp_config& cfg, 
 
 size_t mp_forward_ws(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_params& W) {
     Carve c(nullptr);
+    if (tc_layer(cfg)) {
+        TcBufs t;
+        carve_tc(c, G, cfg, W, false, t);
+        return c.off + 256;
+    }
     LayerFwdBufs b;
     carve_layer(c, G.n_rows, G.n_edges, cfg.hidden, std::max(W.edge.n_lin, W.node.n_lin), false, true, true, b);
     return c.off + 256;
@@ -747,6 +1138,7 @@ int mp_forward(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
                const float* e_in, float* x_out, float* e_out, float* a_star_out, void* ws, size_t ws_bytes,
                cudaStream_t s) {
     GNN_REQUIRE(ws_bytes >= mp_forward_ws(G, cfg, W), GNN_ENOMEM, "gnn_mp_forward: workspace too small");
+    if (tc_layer(cfg)) return tc_mp_forward(G, cfg, W, x_in, e_in, x_out, e_out, a_star_out, ws, s);
     Carve c(ws);
     LayerFwdBufs b;
     carve_layer(c, G.n_rows, G.n_edges, cfg.hidden, std::max(W.edge.n_lin, W.node.n_lin), false, true, true, b);
@@ -783,6 +1175,11 @@ static void carve_bwd(Carve& c, const gnn_graph_dev& G, const gnn_mp_config& cfg
 
 size_t mp_backward_ws(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_params& W) {
     Carve c(nullptr);
+    if (tc_layer(cfg)) {
+        TcBufs t;
+        carve_tc(c, G, cfg, W, true, t);
+        return c.off + 256;
+    }
     LayerFwdBufs b;
     LayerBwdBufs d;
     carve_layer(c, G.n_rows, G.n_edges, cfg.hidden, std::max(W.edge.n_lin, W.node.n_lin), true, true, true, b);
@@ -794,6 +1191,8 @@ int mp_backward(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_p
                 const float* e_in, const float* a_star, const float* dx_out, const float* de_out, float* dx_in,
                 float* de_in, const gnn_mp_params& dW, void* ws, size_t ws_bytes, cudaStream_t s) {
     GNN_REQUIRE(ws_bytes >= mp_backward_ws(G, cfg, W), GNN_ENOMEM, "gnn_mp_backward: workspace too small");
+    if (tc_layer(cfg))
+        return tc_mp_backward(G, cfg, W, x_in, e_in, a_star, dx_out, de_out, dx_in, de_in, dW, ws, s);
     const int H = cfg.hidden;
     const int64_t NR = G.n_rows, E = G.n_edges;
     Carve c(ws);
@@ -875,9 +1274,17 @@ static void carve_mlp(Carve& c, const gnn_mlp& P, int64_t rows, bool bwd, float*
     if (bwd) {
         *g0 = c.take<float>(rows * wmax);
         *g1 = c.take<float>(rows * wmax);
-        *part = c.take<float>((int64_t)partial_floats(P, rows));
+        *part = c.take<float>(tc_widths(P, P.dims[0]) ? tc_grad_floats(P, P.dims[0], 1)
+                                                      : (int64_t)partial_floats(P, rows));
         *dYf = c.take<float>(rows * P.dims[P.n_lin]);
     }
+}
+
+// Linears 0 .. n_lin-2 of a row MLP into h[1 ..].
+static int tc_mlp_hidden(const gnn_mlp& P, int64_t rows, const float* X, float* const* h, cudaStream_t s) {
+    int rc = lin3::run(lin3::kElu, lin_args(rows, X, P.dims[0], P.dims[0], P.W[0], P.dims[0], P.dims[1], P.b[0], h[1],
+                                            P.dims[1]), s);
+    return rc ? rc : tc_hidden(P, rows, h, s);
 }
 
 // The row MLP runs over blocks of at most kMlpRowBlock rows: its workspace
@@ -902,7 +1309,21 @@ int mlp_forward(const gnn_mlp& P, int64_t rows, const float* X, void* Y, int y_b
         Carve c(ws);
         float *h[GNN_MAX_LIN], *z, *g0, *g1, *part, *dy;
         carve_mlp(c, P, n, false, h, &z, &g0, &g1, &part, &dy);
-        int rc = chain_fwd(P, n, X + r0 * K0, K0, h, z, s);
+        int rc;
+        if (tc_widths(P, K0)) {
+            float* out = y_bf16 ? z : (float*)Y + r0 * NO;
+            if ((rc = tc_mlp_hidden(P, n, X + r0 * K0, h, s))) return rc;
+            if ((rc = tc_last(P, n, h, eps, nullptr, out, s))) return rc;
+            if (y_bf16) {
+                {
+                    ProfScope _ps(s, "k_f32_to_bf16");
+                    k_f32_to_bf16<<<grid1(n * NO), 256, 0, s>>>(z, (__nv_bfloat16*)Y + r0 * NO, n * NO);
+                }
+                GNN_LAUNCH_CHECK("k_f32_to_bf16");
+            }
+            continue;
+        }
+        rc = chain_fwd(P, n, X + r0 * K0, K0, h, z, s);
         if (rc) return rc;
         void* Yb = (char*)Y + (size_t)(r0 * NO) * (y_bf16 ? 2 : 4);
         if ((rc = mlp_output(P, n, z, eps, nullptr, nullptr, Yb, y_bf16, s))) return rc;
@@ -920,7 +1341,8 @@ int mlp_backward(const gnn_mlp& P, int64_t rows, const float* X, const void* dY,
         float *h[GNN_MAX_LIN], *z, *g0, *g1, *part, *dyf;
         carve_mlp(c, P, n, true, h, &z, &g0, &g1, &part, &dyf);
         const float* Xb = X + r0 * K0;
-        int rc = chain_fwd(P, n, Xb, K0, h, z, s);
+        const bool tc = tc_widths(P, K0);
+        int rc = tc ? tc_mlp_hidden(P, n, Xb, h, s) : chain_fwd(P, n, Xb, K0, h, z, s);
         if (rc) return rc;
         const float* dy = (const float*)dY + r0 * NO;
         if (dy_bf16) {
@@ -930,6 +1352,18 @@ int mlp_backward(const gnn_mlp& P, int64_t rows, const float* X, const void* dY,
             }
             GNN_LAUNCH_CHECK("k_bf16_to_f32");
             dy = dyf;
+        }
+        if (tc) {
+            GradSums gs(part);
+            const float* dz = nullptr;
+            lin3::Args up{};
+            up.g0 = dy;
+            if ((rc = tc_chain_bwd(P, dP, n, h, eps, up, dy, g0, g1, &dz, gs, s))) return rc;
+            if ((rc = gs.weight(n, dz, P.dims[1], Xb, K0, K0, dP.W[0], K0, dP.b[0], s))) return rc;
+            if ((rc = gs.flush(s))) return rc;
+            if (dX && (rc = lin3::run(lin3::kAdd, dgrad_args(n, dz, P.dims[1], P.W[0], K0, K0, dX + r0 * K0, K0), s)))
+                return rc;
+            continue;
         }
         if ((rc = mlp_bwd(P, dP, n, Xb, K0, h, z, dy, dX ? dX + r0 * K0 : nullptr, g0, g1, part, eps, s)))
             return rc;

@@ -1,4 +1,4 @@
-// Plain FP32 SIMT path of libgnnmp (declarations used by the C-ABI layer).
+// FP32 path of libgnnmp (declarations used by the C-ABI layer).
 #pragma once
 
 #include <cuda_runtime.h>
