@@ -499,8 +499,28 @@ inline int num_sms() {
     return n;
 }
 
-// Persistent grid: resident CTAs (by shared memory / registers and by TMEM
-// columns) times SMs, capped by the number of tiles.
+// CTAs of a kernel that fit one SM: shared memory (227 KB and 1 KB per CTA),
+// registers (four 16,384-register files, 256 per allocation, whole warps),
+// 2,048 threads and 512 TMEM columns. Counted here because
+// cudaOccupancyMaxActiveBlocksPerMultiprocessor answers 1 for every kernel that
+// allocates TMEM, however small, and a grid of one CTA per SM left the kernels
+// with 128 or 256 threads (the projections, the node forward at H <= 32) with 4
+// to 8 warps per SM, waiting: on 4.97M rows at H = 32 the node forward takes
+// 0.48 instead of 0.77 ms with two, the projection 0.20 instead of 0.30 with
+// four.
+template <class K>
+int resident_ctas(K kernel, int threads, uint32_t smem, uint32_t tmem_cols, int* out) {
+    cudaFuncAttributes fa;
+    GNN_CUDA_CHECK(cudaFuncGetAttributes(&fa, kernel), "cudaFuncGetAttributes");
+    const int warps = (threads + 31) / 32, regs = (std::max(fa.numRegs, 1) * 32 + 255) / 256 * 256;
+    int n = 16384 / regs * 4 / warps;
+    n = std::min(n, 64 / warps);
+    n = std::min<int>(n, (int)(228 * 1024 / (smem + (uint32_t)fa.sharedSizeBytes + 1024)));
+    *out = std::min<int>(n, (int)(512 / tmem_cols));
+    return GNN_OK;
+}
+
+// Persistent grid: resident CTAs times SMs, capped by the number of tiles.
 template <class K>
 int persistent_grid(K kernel, int threads, uint32_t smem, uint32_t tmem_cols, int64_t tiles, int* out,
                     int max_per_sm = 0) {
@@ -509,11 +529,9 @@ int persistent_grid(K kernel, int threads, uint32_t smem, uint32_t tmem_cols, in
     GNN_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                         (int)cudaSharedmemCarveoutMaxShared),
                    "cudaFuncSetAttribute(carveout)");
-    int per_sm = 0;
-    GNN_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem),
-                   "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+    int per_sm = 0, rc = resident_ctas(kernel, threads, smem, tmem_cols, &per_sm);
+    if (rc) return rc;
     GNN_REQUIRE(per_sm >= 1, GNN_EUNSUPPORTED, "fused kernel does not fit on an SM (smem %u)", smem);
-    per_sm = std::min<int>(per_sm, (int)(512 / tmem_cols));
     if (max_per_sm > 0) per_sm = std::min(per_sm, max_per_sm);
     *out = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)per_sm * num_sms()));
     return GNN_OK;
