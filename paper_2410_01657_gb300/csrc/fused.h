@@ -89,10 +89,11 @@ int edge_save_tm(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_
 int node_recompute_save(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_params& W,
                         const float* a_star, const float* x_in, RecomputeSave& o, cudaStream_t s);
 
-// Projection adjoint of the BF16 backward: dQ from dz1 over each row's sent
+// Projection adjoint of the BF16 backward: dQ (scratch, [n_rows x H]) from dz1 over each row's sent
 // edges, dx_in += dP W1a + dQ W1b, dW1a and dW1b added into dW.edge.W[0].
 int proj_backward(const gnn_graph_dev& G, int H, const gnn_mp_params& W, const float* x_in, const float* dP,
-                  const __nv_bfloat16* dz1, float* dx_in, const gnn_mp_params& dW, float* part, cudaStream_t s);
+                  const __nv_bfloat16* dz1, __nv_bfloat16* dQ, float* dx_in, const gnn_mp_params& dW, float* part,
+                  cudaStream_t s);
 
 // Layered BF16 backward at H = 128 (recomputation, per-Linear adjoint kernels).
 size_t backward_h128_ws(const gnn_graph_dev& G, const gnn_mp_params& W);

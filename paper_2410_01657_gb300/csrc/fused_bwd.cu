@@ -11,7 +11,7 @@
 //                 back-propagate to de_in = g + W1c^T dz1, write dz1 (the
 //                 gradient of the first pre-activation) per edge, sum it over
 //                 each receiver's edges into dP (FP32, fixed edge order); dW
-//   k_proj_bwd    dQ_j = sum of dz1 over the edges sent by j (sender CSR,
+//   k_sender_sums, k_proj_bwd    dQ_j = sum of dz1 over the edges sent by j (sender CSR,
 //                 fixed order); dx_in += dP W1a + dQ W1b; dW1a, dW1b
 //   k_reduce      per-CTA weight-gradient partials summed in CTA order into dW
 // No atomics anywhere: every sum has a fixed order, so results are bitwise
@@ -102,9 +102,6 @@ struct ProjBwdSmem {
     uint32_t w, a, x, bar, tm, total;
 };
 
-// H = 128 also stages each tile's sender-edge ids (up to kProjEids of them).
-constexpr int kProjEids = 4096;
-
 template <int H>
 __host__ __device__ inline ProjBwdSmem proj_bwd_smem() {
     using C = CfgB<H>;
@@ -112,7 +109,7 @@ __host__ __device__ inline ProjBwdSmem proj_bwd_smem() {
     s.w = 0;
     s.a = align_up(2 * C::WT, 1024);
     s.x = s.a + 2 * C::TILE;
-    s.bar = align_up(s.x + C::TILE + (H == 128 ? kProjEids * 4 : 0), 8);
+    s.bar = align_up(s.x + C::TILE, 8);
     s.tm = s.bar + 16;
     uint32_t end = s.tm + 16;
     end = end > s.a + 32768 ? end : s.a + 32768;
@@ -930,9 +927,7 @@ __global__ void __launch_bounds__(CfgB<H>::NT, 1) k_edge_bwd(const __grid_consta
 struct ProjBwdArgs {
     const float* x;
     const float* dP;
-    const __nv_bfloat16* dz1;
-    const int32_t* t_ptr;
-    const int32_t* t_eid;
+    const __nv_bfloat16* dQ;   // sender-side sums of dz1 (k_sender_sums), as the operand rounds them
     const float* W1;
     float* dx_in;       // += dP W1a + dQ W1b
     float* part;
@@ -940,7 +935,47 @@ struct ProjBwdArgs {
     int64_t n_rows;
 };
 
-// Thread layout: 128 rows x H/32 column groups of 32 columns (two CTAs per SM).
+// dQ_j = sum of dz1 over the edges sent by j, in edge order, FP32, rounded to
+// BF16 once (the operand that k_proj_bwd multiplies). One thread per 8 columns
+// of a row: the gathers of whole 16-byte pieces are the kernel, so it wants
+// every warp the SM holds; inside the projection adjoint (4 to 8 warps per SM
+// at H <= 64, 16 at H = 128) they were a chain of exposed latencies.
+template <int H>
+__global__ void __launch_bounds__(256) k_sender_sums(const int32_t* __restrict__ t_ptr,
+                                                     const int32_t* __restrict__ t_eid,
+                                                     const __nv_bfloat16* __restrict__ dz1, int64_t n_rows,
+                                                     __nv_bfloat16* __restrict__ dQ) {
+    constexpr int PPR = H / 8, UB = 6;   // a lattice node sends to six others
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t r = i / PPR;
+    const int c = (int)(i % PPR) * 8;
+    if (r >= n_rows) return;
+    float dq[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const int32_t k1 = __ldg(t_ptr + r + 1);
+    for (int32_t kb = __ldg(t_ptr + r); kb < k1; kb += UB) {
+        uint4 z[UB];
+#pragma unroll
+        for (int u = 0; u < UB; ++u)
+            z[u] = kb + u < k1 ? __ldg(reinterpret_cast<const uint4*>(dz1 + (int64_t)__ldg(t_eid + kb + u) * H + c))
+                               : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+            if (kb + u < k1) {
+                const uint32_t w[4] = {z[u].x, z[u].y, z[u].z, z[u].w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    float f0, f1;
+                    unpack_bf16x2(w[k], f0, f1);
+                    dq[2 * k] += f0;
+                    dq[2 * k + 1] += f1;
+                }
+            }
+        }
+    }
+    st_bf16x8(dQ + r * H + c, dq);
+}
+
+// Thread layout: 128 rows x H/32 column groups of 32 columns.
 template <int H>
 struct CfgP {
     static constexpr int S = span_of(H);
@@ -998,133 +1033,38 @@ __global__ void __launch_bounds__(CfgP<H>::NT, H >= 128 ? 1 : 2) k_proj_bwd(Proj
             const int64_t nr = std::min<int64_t>(128, A.n_rows - rn);
             prefetch_l2(A.dP + rn * H, (uint32_t)(nr * H * 4));
             prefetch_l2(A.x + rn * H, (uint32_t)(nr * H * 4));
-            if constexpr (H == 128) prefetch_l2(A.dx_in + rn * H, (uint32_t)(nr * H * 4));   // its update
+            prefetch_l2(A.dQ + rn * H, (uint32_t)(nr * H * 2));
+            prefetch_l2(A.dx_in + rn * H, (uint32_t)(nr * H * 4));   // its update
         }
-        const int64_t r = t * 128 + row;
-        const bool valid = r < A.n_rows;
-        if constexpr (H == 128) {
-            // warp-cooperative rows: warp w fills rows 8w .. 8w+7 of the operand tiles, lane l
-            // columns 4l .. 4l+3, so every dz1, dP and x row is one coalesced 256/512-byte read
-            // (the sender-side sum of each column still runs over the edges in order)
-            constexpr int UE = 4;   // edges per row requested together, for all eight rows at once
-            // the tile's sender-edge ids are one contiguous range of t_eid: staged in shared
-            // memory by one coalesced read when it fits, so each gather is a single round trip
-            int32_t* sTe = reinterpret_cast<int32_t*>(sX + 128 * H * 2);
-            const int64_t rt0 = t * 128, rt1 = min(A.n_rows, rt0 + 128);
-            const int32_t kt0 = __ldg(A.t_ptr + rt0), kt1 = __ldg(A.t_ptr + rt1);
-            const bool staged = kt1 - kt0 <= kProjEids;
-            if (staged)
-                for (int i = tid; i < kt1 - kt0; i += C::NT) sTe[i] = __ldg(A.t_eid + kt0 + i);
-            __syncthreads();
-            int32_t k0[8], deg[8];
-            int maxdeg = 0;
+        // the operand tiles [dP dQ] and x, filled by pieces of four columns: consecutive threads
+        // read consecutive pieces, so every global access is a run of whole rows
+        constexpr int PPR = H / 4, IT = 128 * PPR / C::NT, UB = 4;   // pieces per row; steps; steps in flight
+        const int64_t rt = t * 128;
+        const int nv = (int)std::min<int64_t>(128, A.n_rows - rt);
+#pragma unroll 1
+        for (int i0 = 0; i0 < IT; i0 += UB) {
+            float4 dp[UB], xv[UB];
+            uint2 dq[UB];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int64_t rg = t * 128 + 8 * warp + i;
-                k0[i] = rg < A.n_rows ? __ldg(A.t_ptr + rg) : 0;
-                deg[i] = rg < A.n_rows ? __ldg(A.t_ptr + rg + 1) - k0[i] : 0;
-                maxdeg = max(maxdeg, deg[i]);
-            }
-            float4 dq[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) dq[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int kb = 0; kb < maxdeg; kb += UE) {
-                uint2 z[8][UE];
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-#pragma unroll
-                    for (int u = 0; u < UE; ++u) {
-                        const int32_t k = k0[i] + kb + u;
-                        const int64_t e = kb + u < deg[i] ? (int64_t)(staged ? sTe[k - kt0] : __ldg(A.t_eid + k)) : -1;
-                        z[i][u] = e >= 0 ? __ldg(reinterpret_cast<const uint2*>(A.dz1 + e * H) + lane)
-                                         : make_uint2(0u, 0u);
-                    }
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-#pragma unroll
-                    for (int u = 0; u < UE; ++u) {
-                        if (kb + u < deg[i]) {
-                            float f0, f1, f2, f3;
-                            unpack_bf16x2(z[i][u].x, f0, f1);
-                            unpack_bf16x2(z[i][u].y, f2, f3);
-                            dq[i].x += f0;
-                            dq[i].y += f1;
-                            dq[i].z += f2;
-                            dq[i].w += f3;
-                        }
-                    }
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int rr = 8 * warp + i;
-                const int64_t rg = t * 128 + rr;
-                float4 dp = make_float4(0.f, 0.f, 0.f, 0.f), xv = dp;
-                if (rg < A.n_rows) {
-                    dp = __ldg(reinterpret_cast<const float4*>(A.dP + rg * H) + lane);
-                    xv = __ldg(reinterpret_cast<const float4*>(A.x + rg * H) + lane);
-                }
-                *reinterpret_cast<uint2*>(sA + tile_off(rr, H + 4 * lane, 128, S2)) =
-                    make_uint2(pack_bf16x2(dq[i].x, dq[i].y), pack_bf16x2(dq[i].z, dq[i].w));
-                *reinterpret_cast<uint2*>(sA + tile_off(rr, 4 * lane, 128, S2)) =
-                    make_uint2(pack_bf16x2(dp.x, dp.y), pack_bf16x2(dp.z, dp.w));
-                *reinterpret_cast<uint2*>(sX + tile_off(rr, 4 * lane, 128, S)) =
-                    make_uint2(pack_bf16x2(xv.x, xv.y), pack_bf16x2(xv.z, xv.w));
-            }
-        } else {
-            float dq[CW];
-#pragma unroll
-            for (int i = 0; i < CW; ++i) dq[i] = 0.f;
-            if (valid) {
-                // sender-side sum in edge order; the edge ids and then the dz1 rows of UB
-                // edges are requested together so their latencies overlap
-                constexpr int UB = CW >= 32 ? 2 : 4;
-                const int32_t k0 = A.t_ptr[r], k1 = A.t_ptr[r + 1];
-                for (int32_t kb = k0; kb < k1; kb += UB) {
-                    int64_t e[UB];
-#pragma unroll
-                    for (int u = 0; u < UB; ++u) e[u] = kb + u < k1 ? (int64_t)__ldg(A.t_eid + kb + u) : -1;
-                    uint4 z[UB][CW / 8];
-#pragma unroll
-                    for (int u = 0; u < UB; ++u)
-#pragma unroll
-                        for (int i = 0; i < CW / 8; ++i)
-                            z[u][i] = e[u] >= 0 ? __ldg(reinterpret_cast<const uint4*>(A.dz1 + e[u] * H + c0) + i)
-                                                : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                    for (int u = 0; u < UB; ++u) {
-                        if (e[u] < 0) break;
-#pragma unroll
-                        for (int i = 0; i < CW / 8; ++i) {
-                            float f[8];
-                            unpack_bf16x2(z[u][i].x, f[0], f[1]);
-                            unpack_bf16x2(z[u][i].y, f[2], f[3]);
-                            unpack_bf16x2(z[u][i].z, f[4], f[5]);
-                            unpack_bf16x2(z[u][i].w, f[6], f[7]);
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) dq[8 * i + j] += f[j];
-                        }
-                    }
+            for (int u = 0; u < UB; ++u) {
+                const int p = tid + (i0 + u) * C::NT, rr = p / PPR, c = 4 * (p % PPR);
+                dp[u] = xv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                dq[u] = make_uint2(0u, 0u);
+                if (rr < nv) {
+                    const int64_t o = (rt + rr) * H + c;
+                    dp[u] = __ldg(reinterpret_cast<const float4*>(A.dP + o));
+                    xv[u] = __ldg(reinterpret_cast<const float4*>(A.x + o));
+                    dq[u] = __ldg(reinterpret_cast<const uint2*>(A.dQ + o));
                 }
             }
 #pragma unroll
-            for (int i = 0; i < CW; i += 8) st_tile8(sA, row, H + c0 + i, 128, S2, dq + i);
-            {
-                float dp[CW], xv[CW];
-#pragma unroll
-                for (int i = 0; i < CW; ++i) dp[i] = xv[i] = 0.f;
-                if (valid) {
-                    const float4* pp = reinterpret_cast<const float4*>(A.dP + r * H + c0);
-                    const float4* px = reinterpret_cast<const float4*>(A.x + r * H + c0);
-#pragma unroll
-                    for (int i = 0; i < CW / 4; ++i) {
-                        float4 u = __ldg(pp + i), w = __ldg(px + i);
-                        dp[4 * i] = u.x; dp[4 * i + 1] = u.y; dp[4 * i + 2] = u.z; dp[4 * i + 3] = u.w;
-                        xv[4 * i] = w.x; xv[4 * i + 1] = w.y; xv[4 * i + 2] = w.z; xv[4 * i + 3] = w.w;
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < CW; i += 8) st_tile8(sA, row, c0 + i, 128, S2, dp + i);
-                st_row_tile<CW>(sX, row, c0, S, xv);
+            for (int u = 0; u < UB; ++u) {
+                const int p = tid + (i0 + u) * C::NT, rr = p / PPR, c = 4 * (p % PPR);
+                *reinterpret_cast<uint2*>(sA + tile_off(rr, c, 128, S2)) =
+                    make_uint2(pack_bf16x2(dp[u].x, dp[u].y), pack_bf16x2(dp[u].z, dp[u].w));
+                *reinterpret_cast<uint2*>(sA + tile_off(rr, H + c, 128, S2)) = dq[u];
+                *reinterpret_cast<uint2*>(sX + tile_off(rr, c, 128, S)) =
+                    make_uint2(pack_bf16x2(xv[u].x, xv[u].y), pack_bf16x2(xv[u].z, xv[u].w));
             }
         }
         fence_proxy_async();
@@ -1148,39 +1088,31 @@ __global__ void __launch_bounds__(CfgP<H>::NT, H >= 128 ? 1 : 2) k_proj_bwd(Proj
         float d[CW];
         ld_acc<CW>(tWork, q, c0, d);
         tc_fence_before();
-        if constexpr (H == 128) {
-            // dx_in += d as whole rows per warp: the MMAs have read the operand tile, which now
-            // stages the FP32 rows [128 x 128] (row r at 512 r bytes, 16-byte chunks swizzled by r)
-            float4* sD = reinterpret_cast<float4*>(sA);
+        // dx_in += d by the same pieces: the MMAs have read the operand tile, which now stages the
+        // FP32 rows [128 x H] (16-byte pieces swizzled by row)
+        float4* sD = reinterpret_cast<float4*>(sA);
+        constexpr int SWM = PPR >= 8 ? 7 : PPR - 1;
 #pragma unroll
-            for (int i = 0; i < CW / 4; ++i)
-                sD[row * 32 + (((c0 / 4) + i) ^ (row & 7))] = make_float4(d[4 * i], d[4 * i + 1], d[4 * i + 2], d[4 * i + 3]);
-            __syncthreads();
-#pragma unroll 4
-            for (int i = 0; i < 8; ++i) {
-                const int rr = 8 * warp + i;
-                const int64_t rg = t * 128 + rr;
-                if (rg < A.n_rows) {
-                    float4* po = reinterpret_cast<float4*>(A.dx_in + rg * H) + lane;
-                    const float4 v = sD[rr * 32 + (lane ^ (rr & 7))];
-                    float4 o = *po;
-                    o.x += v.x;
-                    o.y += v.y;
-                    o.z += v.z;
-                    o.w += v.w;
-                    *po = o;
-                }
+        for (int i = 0; i < CW / 4; ++i)
+            sD[row * PPR + (((c0 / 4) + i) ^ (row & SWM))] =
+                make_float4(d[4 * i], d[4 * i + 1], d[4 * i + 2], d[4 * i + 3]);
+        __syncthreads();
+#pragma unroll 1
+        for (int i0 = 0; i0 < IT; i0 += UB) {
+            float4 o[UB];
+#pragma unroll
+            for (int u = 0; u < UB; ++u) {
+                const int p = tid + (i0 + u) * C::NT, rr = p / PPR;
+                if (rr < nv) o[u] = *(reinterpret_cast<const float4*>(A.dx_in + rt * H) + p);
             }
-        } else if (valid) {
-            float4* po = reinterpret_cast<float4*>(A.dx_in + r * H + c0);
 #pragma unroll
-            for (int i = 0; i < CW / 4; ++i) {
-                float4 o = po[i];
-                o.x += d[4 * i];
-                o.y += d[4 * i + 1];
-                o.z += d[4 * i + 2];
-                o.w += d[4 * i + 3];
-                po[i] = o;
+            for (int u = 0; u < UB; ++u) {
+                const int p = tid + (i0 + u) * C::NT, rr = p / PPR, c = p % PPR;
+                if (rr < nv) {
+                    const float4 v = sD[rr * PPR + (c ^ (rr & SWM))];
+                    *(reinterpret_cast<float4*>(A.dx_in + rt * H) + p) =
+                        make_float4(o[u].x + v.x, o[u].y + v.y, o[u].z + v.z, o[u].w + v.w);
+                }
             }
         }
         first = false;
@@ -1310,20 +1242,24 @@ BwdWs carve_bwd(void* ws, const gnn_graph_dev& G, int H, int Le, int Ln, bool ne
 
 template <int H>
 int proj_backward_h(const gnn_graph_dev& G, const gnn_mp_params& W, const float* x_in, const float* dP,
-                    const __nv_bfloat16* dz1, float* dx_in, const gnn_mp_params& dW, float* part, cudaStream_t s) {
+                    const __nv_bfloat16* dz1, __nv_bfloat16* dQ, float* dx_in, const gnn_mp_params& dW, float* part,
+                    cudaStream_t s) {
     const int64_t NR = G.n_rows;
     if (NR == 0) return GNN_OK;
     ProjBwdArgs A;
     A.x = x_in;
     A.dP = dP;
-    A.dz1 = dz1;
-    A.t_ptr = G.t_ptr;
-    A.t_eid = G.t_eid;
+    A.dQ = dQ;
     A.W1 = W.edge.W[0];
     A.dx_in = dx_in;
     A.part = part;
     A.pstride = proj_pstride(H);
     A.n_rows = NR;
+    {
+        ProfScope _ps(s, "k_sender_sums");
+        k_sender_sums<H><<<(unsigned)((NR * (H / 8) + 255) / 256), 256, 0, s>>>(G.t_ptr, G.t_eid, dz1, NR, dQ);
+    }
+    GNN_LAUNCH_CHECK("k_sender_sums");
     const ProjBwdSmem P = proj_bwd_smem<H>();
     int grid;
     int rc = persistent_grid(k_proj_bwd<H>, CfgP<H>::NT, P.total, pow2_cols(2 * H > 128 ? 3 * H : 2 * H),
@@ -1478,7 +1414,7 @@ int backward_h(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
         GNN_CUDA_CHECK(cudaMemsetAsync(w.dP, 0, sizeof(float) * NR * H, s), "memset");
     }
     // 4. projection adjoint: sender-side sums, dx_in += [dP dQ] [W1a; W1b], dW1a, dW1b
-    return proj_backward_h<H>(G, W, x_in, w.dP, w.dz1, dx_in, dW, w.part, s);
+    return proj_backward_h<H>(G, W, x_in, w.dP, w.dz1, w.pq, dx_in, dW, w.part, s);   // (P|Q is done with)
 }
 
 }  // namespace
@@ -1489,12 +1425,13 @@ size_t mp_backward_ws(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gn
 }
 
 int proj_backward(const gnn_graph_dev& G, int H, const gnn_mp_params& W, const float* x_in, const float* dP,
-                  const __nv_bfloat16* dz1, float* dx_in, const gnn_mp_params& dW, float* part, cudaStream_t s) {
+                  const __nv_bfloat16* dz1, __nv_bfloat16* dQ, float* dx_in, const gnn_mp_params& dW, float* part,
+                  cudaStream_t s) {
     switch (H) {
-        case 16: return proj_backward_h<16>(G, W, x_in, dP, dz1, dx_in, dW, part, s);
-        case 32: return proj_backward_h<32>(G, W, x_in, dP, dz1, dx_in, dW, part, s);
-        case 64: return proj_backward_h<64>(G, W, x_in, dP, dz1, dx_in, dW, part, s);
-        case 128: return proj_backward_h<128>(G, W, x_in, dP, dz1, dx_in, dW, part, s);
+        case 16: return proj_backward_h<16>(G, W, x_in, dP, dz1, dQ, dx_in, dW, part, s);
+        case 32: return proj_backward_h<32>(G, W, x_in, dP, dz1, dQ, dx_in, dW, part, s);
+        case 64: return proj_backward_h<64>(G, W, x_in, dP, dz1, dQ, dx_in, dW, part, s);
+        case 128: return proj_backward_h<128>(G, W, x_in, dP, dz1, dQ, dx_in, dW, part, s);
         default: return set_error(GNN_EUNSUPPORTED, "proj_backward: H=%d", H);
     }
 }
