@@ -79,12 +79,13 @@ int gnn_check(void* stream) {
     GNN_CUDA_CHECK(cudaStreamSynchronize((cudaStream_t)stream), "gnn_check: stream synchronize");
     // every translation unit with waiting kernels has its own error word
     cudaError_t (*const take[])(unsigned int*) = {
-        gnn::plain::take_device_error, gnn::lin3::take_device_error, gnn::fused::take_device_error, gnn::fused::take_device_error_bwd,
+        gnn::plain::take_device_error, gnn::lin3::take_device_error, gnn::fused::take_device_error,
+        gnn::fused::take_device_error_bwd, gnn::fused::take_device_error_edge_bwd,
         gnn::fused::take_device_error_bwd128, gnn::fused::take_device_error_rowmlp,
         gnn::fused::take_device_error_edge128, gnn::fused::take_device_error_rowenc128,
         gnn::fused::take_device_error_rowdec128, gnn::fused::take_device_error_node128,
         gnn::diag::take_device_error};
-    const char* const unit[] = {"plain", "lin3", "fused", "fused_bwd", "bwd128", "rowmlp", "edge128", "rowenc128",
+    const char* const unit[] = {"plain", "lin3", "fused", "fused_bwd", "edge_bwd", "bwd128", "rowmlp", "edge128", "rowenc128",
                                 "rowdec128", "node128", "diag"};
     static_assert(sizeof(unit) / sizeof(unit[0]) == sizeof(take) / sizeof(take[0]), "one name per unit");
     unsigned int word = 0;

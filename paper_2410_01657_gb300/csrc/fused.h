@@ -9,10 +9,11 @@
 namespace gnn {
 namespace fused {
 
-// Read and clear the device error word of fused.cu, fused_bwd.cu, bwd128.cu, rowmlp.cu, edge128.cu,
+// Read and clear the device error word of fused.cu, fused_bwd.cu, edge_bwd.cu, bwd128.cu, rowmlp.cu, edge128.cu,
 // rowenc128.cu, rowdec128.cu, node128.cu.
 cudaError_t take_device_error(unsigned int* out);
 cudaError_t take_device_error_bwd(unsigned int* out);
+cudaError_t take_device_error_edge_bwd(unsigned int* out);
 cudaError_t take_device_error_bwd128(unsigned int* out);
 cudaError_t take_device_error_rowmlp(unsigned int* out);
 cudaError_t take_device_error_edge128(unsigned int* out);
@@ -88,6 +89,26 @@ int edge_save_tm(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_
                  const __nv_bfloat16* pq, RecomputeSave& o, cudaStream_t s);
 int node_recompute_save(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_params& W,
                         const float* a_star, const float* x_in, RecomputeSave& o, cudaStream_t s);
+
+// Edge adjoint at H <= 64 (edge_bwd.cu): de_in, dz_0 per edge, its receiver sums
+// dP, and per-CTA partials (pstride apart, *grid of them, at most one per SM): per
+// layer [H x (H + 16)], bias gradients in column H, then dgamma, dbeta.
+struct EdgeBackward {
+    const __nv_bfloat16* pq;      // P rows, then Q rows (not read with act)
+    const float* da;
+    const __nv_bfloat16* e_in;
+    const __nv_bfloat16* de_out;  // NULL: zero
+    const __nv_bfloat16* act;     // saved hidden activations, or NULL: recomputed
+    __nv_bfloat16* de_in;
+    __nv_bfloat16* dz1;
+    float* dP;
+    float* part;
+    int64_t pstride;
+    float eps;
+};
+bool edge_backward_supported(int H, int n_lin);
+int edge_backward(const gnn_graph_dev& G, int H, const gnn_mp_params& W, const EdgeBackward& o, int* grid,
+                  cudaStream_t s);
 
 // Projection adjoint of the BF16 backward: dQ (scratch, [n_rows x H]) from dz1 over each row's sent
 // edges, dx_in += dP W1a + dQ W1b, dW1a and dW1b added into dW.edge.W[0].

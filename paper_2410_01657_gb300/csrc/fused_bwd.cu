@@ -39,40 +39,6 @@ cudaError_t take_device_error_bwd(unsigned int* out) { return take_device_error_
 
 // ------------------------------------------------------------------ shared memory plans
 
-struct EdgeBwdSmem {
-    uint32_t w, e0, de, g, hb, ones, slot, par, seg, red, bar, tm, total;
-};
-
-// Edge-backward shared memory. g holds the tile's dz rows during the adjoint
-// and, during the recompute, the aggregate gradients da of the tile's
-// receivers (when they fit: nr * H * 4 <= TILE). hb holds the recomputed
-// hidden activations and, once the adjoint no longer reads them, the staging
-// of the segmented sum dP. slot: the next tile's P rows [128 x H], then each
-// thread's Q columns for it.
-template <int H>
-__host__ __device__ inline EdgeBwdSmem edge_bwd_smem(int n_lin) {
-    using C = CfgB<H>;
-    EdgeBwdSmem s;
-    s.w = 0;
-    s.e0 = align_up(n_lin * C::WT, 1024);         // 2 stages of {e tile, de tile}
-    s.de = s.e0 + C::TILE;
-    s.seg = s.e0 + 4 * C::TILE;                    // 2 tile records (GNN_TILE_META_BYTES each)
-    s.g = align_up(s.seg + 2 * GNN_TILE_META_BYTES, 1024);
-    s.hb = s.g + C::TILE;
-    const uint32_t hb_min = 128 * H * 4, hb_tiles = (uint32_t)(n_lin - 1) * C::TILE;
-    const uint32_t hb_bytes = hb_tiles > hb_min ? hb_tiles : hb_min;
-    s.ones = align_up(s.hb + hb_bytes, 1024);
-    s.slot = align_up(s.ones + 128 * C::S, 1024);
-    s.par = s.slot + 2 * C::TILE;
-    s.red = s.par + (n_lin + 2) * H * 4;
-    s.bar = align_up(s.red + 4 * C::CG * 128 * 4, 8);   // full[2], mma, ready, da, wgrad, P rows, h[GNN_MAX_LIN]
-    s.tm = s.bar + 8 * (7 + GNN_MAX_LIN);
-    uint32_t end = s.tm + 16;
-    end = end > s.g + 32768 ? end : s.g + 32768;   // M-padded wgrad views read 32 KB from g
-    s.total = end + 1024;
-    return s;
-}
-
 struct NodeBwdSmem {
     uint32_t w0, w, ain, ones2, g, hb, ones, par, red, bar, tm, total;
 };
@@ -118,11 +84,6 @@ __host__ __device__ inline ProjBwdSmem proj_bwd_smem() {
 }
 
 // TMEM column plans
-template <int H>
-__host__ __device__ inline uint32_t edge_bwd_tcols(int n_lin) { return H + n_lin * (H + 16); }
-// ... plus the LayerNorm parameter-gradient accumulators (2H columns) when they fit
-template <int H>
-__host__ __device__ inline bool edge_bwd_ln_in_tmem(int n_lin) { return edge_bwd_tcols<H>(n_lin) + 2 * H <= 512; }
 // Offset of the LayerNorm parameter gradients in a node-adjoint CTA's partials
 // (after the weight-gradient blocks [H x (2H+16)] and (n_lin-1) x [H x (H+16)]).
 template <int H>
@@ -153,7 +114,7 @@ struct NodeBwdArgs {
 // SAVED: the forward stored the node MLP's hidden activations (block k, row
 // k * act_rows + r, of tmap_h) and its BF16 input rows [a*, x] (tmap_xa); they
 // arrive by TMA into the activation buffers and the input tile, each refilled
-// with the next tile's rows once its last reader has passed (as in k_edge_bwd),
+// with the next tile's rows once its last reader has passed (as in the edge adjoint),
 // and only the last Linear is recomputed; a* and x are not read.
 template <int H, bool SAVED>
 __global__ void __launch_bounds__(CfgB<H>::NT, 1) k_node_bwd(const __grid_constant__ CUtensorMap tmap_h,
@@ -224,7 +185,7 @@ __global__ void __launch_bounds__(CfgB<H>::NT, 1) k_node_bwd(const __grid_consta
     uint32_t ph = 0, ph_w = 0, ph_rdy = 0;
     bool ok = true, first = true;
     const int64_t n_tiles = (A.n_rows + 127) / 128;
-    // MMA hand-off as in k_edge_bwd: warps arrive on `ready` after their operand writes and
+    // MMA hand-off as in the edge adjoint: warps arrive on `ready` after their operand writes and
     // accumulator reads, thread 0 issues, every thread waits on the completion barrier itself
     auto handoff = [&](auto&& issue, uint64_t* done) {
         fence_proxy_async();
@@ -444,478 +405,6 @@ __global__ void __launch_bounds__(CfgB<H>::NT, 1) k_node_bwd(const __grid_consta
     }
     colsum_store<H, NCH>(acc_g, sRed, q, lane, c0, tid, C::NT, part + node_ln_off<H>(L));
     colsum_store<H, NCH>(acc_b, sRed, q, lane, c0, tid, C::NT, part + node_ln_off<H>(L) + H);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (warp == 0) tmem_dealloc(tmem, NCOLS);
-}
-
-// ------------------------------------------------------------------ k_edge_bwd
-
-struct EdgeBwdArgs {
-    const uint8_t* tile_meta;   // per-tile records (GNN_TILE_META_BYTES each)
-    int64_t n_tiles;
-    const __nv_bfloat16* pq;    // P rows [n_rows x H]
-    const __nv_bfloat16* q;     // Q rows [n_rows x H]
-    const float* da;            // gradient of the aggregate after the halo adjoint
-    int has_de_out;
-    __nv_bfloat16* de_in;
-    __nv_bfloat16* dz1;         // per-edge gradient of the first pre-activation
-    float* dP;                  // per-row sum of dz1 over the row's received edges
-    float* part;
-    int64_t pstride;
-    MlpDev mlp;
-    float eps;
-    int64_t act_rows;           // SAVED: rows of one activation block of tmap_h (tiles * 128)
-};
-
-// LNT: the per-thread LayerNorm gradient sums live in TMEM columns after the
-// weight-gradient accumulators (read, add, write back once per tile) instead
-// of 2*CW registers.
-// SAVED: the forward stored the hidden activations h_0 .. h_{L-2} of every edge
-// (row k * act_rows + t * 128 + i of tmap_h for edge row i of tile t); the tile's rows arrive by TMA into the
-// activation buffers and only the last Linear is recomputed (no P|Q gather, no
-// ELU chain). Buffer k is refilled with the next tile's rows as soon as the
-// adjoint step that reads it last has passed its hand-off, so the loads have
-// most of a tile's time to land; the dP staging moves to the P|Q slot area.
-template <int H, bool LNT, bool SAVED>
-__global__ void __launch_bounds__(CfgB<H>::NT, 1) k_edge_bwd(const __grid_constant__ CUtensorMap tmap_e,
-                                                            const __grid_constant__ CUtensorMap tmap_de,
-                                                            const __grid_constant__ CUtensorMap tmap_h,
-                                                            EdgeBwdArgs A) {
-    using C = CfgB<H>;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* sm = aligned_smem(smem_raw);
-    const int L = A.mlp.n_lin;
-    const EdgeBwdSmem P = edge_bwd_smem<H>(L);
-    uint8_t* sW = sm + P.w;
-    uint8_t* sStg0 = sm + P.e0;       // stage s: e tile at +2*s*TILE, de tile right after it
-    uint8_t* sRec0 = sm + P.seg;      // stage s: tile record at +s*GNN_TILE_META_BYTES
-    uint8_t* sG = sm + P.g;
-    uint8_t* sHB = sm + P.hb;
-    uint8_t* sOnes = sm + P.ones;
-    float* sStage = reinterpret_cast<float*>(SAVED ? sm + P.slot : sHB);   // dP staging at the last adjoint step
-    float* sPar = reinterpret_cast<float*>(sm + P.par);
-    float* sRed = reinterpret_cast<float*>(sm + P.red);
-    uint64_t* full = reinterpret_cast<uint64_t*>(sm + P.bar);   // full[2]: stage loaded
-    uint64_t* bar = full + 2;       // MMA completion
-    uint64_t* ready = full + 3;     // one arrival per warp: operands written, accumulator read
-    uint64_t* da_full = full + 4;   // the tile's da rows have landed in sG
-    uint64_t* bar_w = full + 5;     // weight-gradient MMAs of an adjoint step (complete behind the epilogue)
-    uint64_t* p_full = full + 6;    // the tile's P rows have landed in sP
-    uint64_t* h_full = full + 7;    // SAVED: h_k of the tile has landed in sHB + k * TILE
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + P.tm);
-    constexpr int S = C::S, CW = C::CW;
-    const uint32_t NCOLS = pow2_cols(edge_bwd_tcols<H>(L) + (LNT ? 2 * H : 0));
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int q = warp & 3, g = warp >> 2, row = 32 * q + lane, c0 = g * CW;
-    constexpr int NCH = 2 * CW / 16;                               // 16-byte chunks of a Q slot
-    uint8_t* sP = sm + P.slot;                                     // P rows of the tile's receivers
-    uint8_t* sSlot = sm + P.slot + C::TILE + (g * 128 + row) * (2 * CW);
-    auto slot_at = [&](int k) { return sSlot + 16 * (k ^ ((row >> (NCH >= 8 ? 0 : (NCH == 4 ? 1 : 2))) & (NCH - 1))); };
-
-    if (warp == 0) {
-        tmem_alloc(tslot, NCOLS);
-        tmem_relinquish();
-    }
-    if (tid == 0) {
-        mbar_init(full, 1);
-        mbar_init(full + 1, 1);
-        mbar_init(bar, 1);
-        mbar_init(ready, C::NT / 32);
-        mbar_init(da_full, 1);
-        mbar_init(bar_w, 1);
-        mbar_init(p_full, 1);
-        if (SAVED)
-            for (int k = 0; k < L - 1; ++k) mbar_init(h_full + k, 1);
-        fence_mbar_init();
-    }
-    load_weight(sW, A.mlp.W[0], 3 * H, 2 * H, H, H, tid, C::NT);
-    for (int k = 1; k < L; ++k) load_weight(sW + k * C::WT, A.mlp.W[k], H, 0, H, H, tid, C::NT);
-    fill_ones(sOnes, S, tid, C::NT);
-    for (int i = tid; i < L * H; i += C::NT) sPar[i] = A.mlp.b[i / H][i % H];
-    for (int i = tid; i < H; i += C::NT) {
-        sPar[L * H + i] = A.mlp.gamma[i];
-        sPar[(L + 1) * H + i] = A.mlp.beta[i];
-    }
-    fence_proxy_async();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tslot;
-    const uint32_t tWork = tmem;
-    auto tDW = [&](int k) -> uint32_t { return tmem + (uint32_t)(H + k * (H + 16)); };
-    const uint32_t ones_addr = smem_u32(sOnes);
-    // LayerNorm gradient sums sum_rows g * xhat and sum_rows g: in TMEM (LNT, one lane per
-    // row), else as per-warp column sums (warp_colsum16, one register per 16 columns)
-    constexpr int ACW = LNT ? 1 : CW / 16;
-    float acc_g[ACW], acc_b[ACW];
-#pragma unroll
-    for (int i = 0; i < ACW; ++i) acc_g[i] = acc_b[i] = 0.f;
-    const uint32_t tLN = tmem + ((uint32_t)(32 * q) << 16) + edge_bwd_tcols<H>(L) + (uint32_t)(g * 2 * CW);
-    if constexpr (LNT) {
-        float z[16] = {};
-#pragma unroll
-        for (int i = 0; i < 2 * CW; i += 16) tmem_st16(tLN + i, z);
-        tmem_st_wait();
-    }
-    uint32_t ph = 0, ph_rdy = 0, ph_da = 0, ph_w = 0, ph_p = 0;
-    bool ok = true, first = true;
-    // MMA hand-off without block barriers: every warp arrives on `ready` once its
-    // operand writes and its TMEM reads of the accumulator are done; thread 0
-    // waits for all warps, issues and commits to `bar`; every thread waits on
-    // `bar` by itself. After a timeout a thread stops waiting and issuing; the
-    // block leaves the tile loop together at the tile-end barrier.
-    auto handoff = [&](auto&& issue, uint64_t* done) {
-        fence_proxy_async();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(ready);
-        if (tid == 0) {
-            ok = ok && mbar_wait(ready, ph_rdy);
-            ph_rdy ^= 1;
-            tc_fence_after();
-            if (ok) {
-                issue();
-                mma_commit(done);
-            }
-        }
-    };
-    auto mma_wait = [&]() {
-        ok = ok && mbar_wait(bar, ph);
-        ph ^= 1;
-        __syncwarp();
-        tc_fence_after();
-    };
-    const uint32_t tx_bytes = C::TILE * (A.has_de_out ? 2 : 1) + GNN_TILE_META_BYTES;
-    // stage s <- tile t: its record by bulk copy, its e (and de_out) rows by TMA
-    // (e0: the tile's first edge, read from its global record one tile in advance)
-    auto issue_stage = [&](int s, int64_t t, int32_t e0) {
-        uint8_t* rec = sRec0 + s * GNN_TILE_META_BYTES;
-        uint8_t* se = sStg0 + s * 2 * C::TILE;
-        mbar_arrive_expect_tx(full + s, tx_bytes);
-        bulk_load(rec, A.tile_meta + t * GNN_TILE_META_BYTES, GNN_TILE_META_BYTES, full + s);
-        tma_load_2d(se, &tmap_e, 0, e0, full + s);
-        if (A.has_de_out) tma_load_2d(se + C::TILE, &tmap_de, 0, e0, full + s);
-    };
-    // the receivers' P rows of the tile whose record is in stage s: one bulk copy of the
-    // tile's consecutive rows (thread 0); this thread's Q slot <- the Q row of its edge's
-    // sender, own columns, by cp.async
-    bool p_pending = false;   // thread 0: a P copy not yet consumed (waited for before exit)
-    auto fetch_p = [&](int s) {
-        p_pending = true;
-        const int32_t* hdr = reinterpret_cast<const int32_t*>(sRec0 + s * GNN_TILE_META_BYTES);
-        const int32_t nr = min(max(hdr[1] - hdr[0], 0), 128);   // a tile has 1..128 rows
-        const uint32_t bytes = (uint32_t)nr * H * 2;
-        if (bytes == 0) {
-            mbar_arrive(p_full);
-            return;
-        }
-        mbar_arrive_expect_tx(p_full, bytes);
-        bulk_load(sP, A.pq + (int64_t)hdr[0] * H, bytes, p_full);
-    };
-    auto gather = [&](int s) {
-        const uint8_t* rec = sRec0 + s * GNN_TILE_META_BYTES;
-        if (row < reinterpret_cast<const int32_t*>(rec)[3]) {
-            const int64_t snd = reinterpret_cast<const int32_t*>(rec + 800)[row];
-#pragma unroll
-            for (int k = 0; k < NCH; ++k) cp_async16(slot_at(k), A.q + snd * H + c0 + 8 * k);
-        }
-        cp_async_commit();
-        if (tid == 0) fetch_p(s);
-    };
-    auto first_edge = [&](int64_t t) { return ld_nc_s32(A.tile_meta + t * GNN_TILE_META_BYTES + 8); };
-    // SAVED: h_k rows of the tile starting at edge eh into buffer k (thread 0); per-thread
-    // parity bit k of h_full[k] (one phase per tile); thread 0's loads not yet waited for
-    const uint32_t hmask = SAVED ? ((1u << (L - 1)) - 1u) : 0u;
-    uint32_t ph_h = 0, h_pend = 0;
-    auto load_h = [&](int k, int64_t tt) {
-        mbar_arrive_expect_tx(h_full + k, C::TILE);
-        tma_load_2d(sHB + k * C::TILE, &tmap_h, 0, (int32_t)(k * A.act_rows + tt * 128), h_full + k);
-        h_pend |= 1u << k;
-    };
-    auto wait_h = [&](int k) {
-        ok = ok && mbar_wait(h_full + k, (ph_h >> k) & 1u);
-        h_pend &= ~(1u << k);
-    };
-    int32_t e0_next = 0;   // thread 0: first edge of the CTA's next tile
-    if (tid == 0 && (int64_t)blockIdx.x < A.n_tiles) {
-        issue_stage(0, blockIdx.x, first_edge(blockIdx.x));
-        if (SAVED)
-            for (int k = 0; k < L - 1; ++k) load_h(k, blockIdx.x);
-        if ((int64_t)blockIdx.x + gridDim.x < A.n_tiles) e0_next = first_edge(blockIdx.x + gridDim.x);
-    }
-    if ((int64_t)blockIdx.x < A.n_tiles) {
-        ok = mbar_wait(full, 0);
-        if (ok && !SAVED) gather(0);
-    }
-    int j = 0;
-
-    for (int64_t t = blockIdx.x; t < A.n_tiles; t += gridDim.x, ++j) {
-        const int st = j & 1;
-        ok = ok && mbar_wait(full + st, (uint32_t)(j >> 1) & 1u);
-        __syncwarp();
-        const uint8_t* rec = sRec0 + st * GNN_TILE_META_BYTES;
-        const int32_t* hdr = reinterpret_cast<const int32_t*>(rec);
-        const int32_t* sRp = reinterpret_cast<const int32_t*>(rec + 16);
-        const int16_t* sSeg = reinterpret_cast<const int16_t*>(rec + 544);
-        const float* sW1d = reinterpret_cast<const float*>(rec + 1312);
-        uint8_t* sE0 = sStg0 + st * 2 * C::TILE;
-        uint8_t* sDE = sE0 + C::TILE;
-        const int32_t r0 = hdr[0], r1 = hdr[1], e0 = hdr[2], ne = hdr[3];
-        const bool valid = row < ne;
-        const int64_t eg = (int64_t)e0 + row;
-        // the receivers' da rows into sG for the LayerNorm adjoint (sG is free until then)
-        const bool da_bulk = (r1 - r0) * H * 4 <= C::TILE;
-        if (tid == 0 && ok && da_bulk) {
-            mbar_arrive_expect_tx(da_full, (uint32_t)(r1 - r0) * H * 4);
-            bulk_load(sG, A.da + (int64_t)r0 * H, (uint32_t)(r1 - r0) * H * 4, da_full);
-        }
-        if (tid == 0 && ok) {
-            if (SAVED) wait_h(L - 2);
-            tc_fence_after();
-            if (ok) {
-                if (SAVED) issue_mma(tWork, sHB + (L - 2) * C::TILE, sW + (L - 1) * C::WT, H, H);
-                else issue_mma(tWork, sE0, sW, H, H);
-                mma_commit(bar);
-            }
-            // the other stage was released at the end of the previous tile: prefetch the next tile
-            if (t + gridDim.x < A.n_tiles) {
-                issue_stage(st ^ 1, t + gridDim.x, e0_next);
-                if (t + 2 * (int64_t)gridDim.x < A.n_tiles) e0_next = first_edge(t + 2 * (int64_t)gridDim.x);
-            }
-        }
-        // ---- recompute the chain (SAVED: only the last Linear, from the saved h_{L-2})
-        float v[CW];
-        if constexpr (SAVED) {
-            mma_wait();
-            ld_acc<CW>(tWork, q, c0, v);
-            add_bias2<CW>(v, sPar + (L - 1) * H + c0);
-        }
-        if constexpr (!SAVED) cp_async_wait_all();   // this thread's P|Q slot for the tile
-        for (int k = 0; k < (SAVED ? 0 : L); ++k) {
-            mma_wait();
-            ld_acc<CW>(tWork, q, c0, v);
-            if (k == 0) {
-                ok = ok && mbar_wait(p_full, ph_p);   // the tile's P rows
-                ph_p ^= 1;
-                p_pending = false;
-                if (valid) {
-                    const uint8_t* prow = sP + (int)sSeg[row] * (2 * H) + 2 * c0;
-#pragma unroll
-                    for (int kc = 0; kc < NCH; ++kc) {
-                        const uint4 up = *reinterpret_cast<const uint4*>(prow + 16 * kc);
-                        const uint4 uq = *reinterpret_cast<const uint4*>(slot_at(kc));
-                        const uint32_t pw[4] = {up.x, up.y, up.z, up.w}, qw[4] = {uq.x, uq.y, uq.z, uq.w};
-#pragma unroll
-                        for (int h = 0; h < 4; ++h) {
-                            float p0, p1, q0, q1;
-                            unpack_bf16x2(pw[h], p0, p1);
-                            unpack_bf16x2(qw[h], q0, q1);
-                            const float2 t2 = __fadd2_rn(__fadd2_rn(make_float2(p0, p1), make_float2(q0, q1)),
-                                                         *reinterpret_cast<const float2*>(sPar + c0 + 8 * kc + 2 * h));
-                            float2* vv = reinterpret_cast<float2*>(v + 8 * kc + 2 * h);
-                            *vv = __fadd2_rn(*vv, t2);
-                        }
-                    }
-                } else {
-                    add_bias2<CW>(v, sPar + c0);
-                }
-
-            } else {
-                add_bias2<CW>(v, sPar + k * H + c0);
-            }
-            if (k < L - 1) {
-                elu_inplace2<CW>(v);
-                st_row_tile<CW>(sHB + k * C::TILE, row, c0, S, v);
-                handoff([&] { issue_mma(tWork, sHB + k * C::TILE, sW + (k + 1) * C::WT, H, H); }, bar);
-            }
-        }
-        tc_fence_before();
-        // ---- gradient of e' (adjoint of Eq. 5b plus the upstream edge gradient)
-        float gv[CW];
-        if (da_bulk) {
-            ok = ok && mbar_wait(da_full, ph_da);
-            ph_da ^= 1;
-        }
-        if (valid) {
-            float dar[CW];
-            const float* src = da_bulk ? reinterpret_cast<const float*>(sG) + (int64_t)sSeg[row] * H + c0
-                                       : A.da + (int64_t)(r0 + sSeg[row]) * H + c0;
-#pragma unroll
-            for (int i = 0; i < CW / 4; ++i) {
-                const float4 u = *reinterpret_cast<const float4*>(src + 4 * i);
-                dar[4 * i] = u.x; dar[4 * i + 1] = u.y; dar[4 * i + 2] = u.z; dar[4 * i + 3] = u.w;
-            }
-            const float w = sW1d[row];
-            float deo[CW];
-            if (A.has_de_out) ld_row_tile<CW>(sDE, row, c0, S, deo);
-#pragma unroll
-            for (int i = 0; i < CW; ++i) gv[i] = (A.has_de_out ? deo[i] : 0.f) + w * dar[i];
-        } else {
-#pragma unroll
-            for (int i = 0; i < CW; ++i) gv[i] = 0.f;
-        }
-        // ---- LayerNorm adjoint (statistics and adjoint sums in one exchange)
-        float dz[CW];
-#pragma unroll
-        for (int i = 0; i < CW; ++i) dz[i] = gv[i] * sPar[L * H + c0 + i];
-        float mean, rstd, s1, s2;
-        row_stats_adj<H, C::CG, CW>(v, dz, sRed, row, g, A.eps, mean, rstd, s1, s2);
-#pragma unroll
-        for (int i = 0; i < CW; ++i) v[i] = (v[i] - mean) * rstd;   // xhat
-        if constexpr (LNT) {
-#pragma unroll
-            for (int i0 = 0; i0 < CW; i0 += 16) {
-                float ag[16], ab[16];
-                tmem_ld16(tLN + i0, ag);
-                tmem_ld16(tLN + CW + i0, ab);
-                tmem_ld_wait();
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    ag[i] += gv[i0 + i] * v[i0 + i];
-                    ab[i] += gv[i0 + i];
-                }
-                tmem_st16(tLN + i0, ag);
-                tmem_st16(tLN + CW + i0, ab);
-            }
-            tmem_st_wait();
-        } else {
-#pragma unroll
-            for (int j = 0; j < ACW; ++j) {
-                float t16[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) t16[i] = gv[16 * j + i] * v[16 * j + i];
-                acc_g[j] += warp_colsum16(t16, lane);
-                acc_b[j] += warp_colsum16(gv + 16 * j, lane);
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < CW; ++i) dz[i] = rstd * (dz[i] - s1 - v[i] * s2);
-        // ---- chain adjoint
-        for (int k = L - 1; k >= 0; --k) {
-            if (k < L - 1) {   // the previous step's wgrad reads sG: wait for it (per thread, no barrier)
-                ok = ok && mbar_wait(bar_w, ph_w);
-                ph_w ^= 1;
-            }
-            if (SAVED && k > 0) wait_h(k - 1);   // this step's wgrad operand and ELU derivative input
-            st_row_tile<CW>(sG, row, c0, S, dz);
-            handoff([&] {
-                issue_dgrad(tWork, sG, S, sW + k * C::WT, S, H, (uint32_t)H * S, H, H);
-                mma_commit(bar);
-                uint8_t* hk = (k == 0) ? sE0 : sHB + (k - 1) * C::TILE;
-                issue_wgrad(tDW(k), sG, S, 128u * S, hk, S, ones_addr - smem_u32(hk), H + 16, !first);
-            }, bar_w);
-            // SAVED: every thread has passed its last read of h_k (step k + 1) and its wgrad has
-            // completed (bar_w, waited at the top of this step): the next tile's h_k goes there
-            if (SAVED && tid == 0 && ok && k <= L - 2 && t + gridDim.x < A.n_tiles) load_h(k, t + gridDim.x);
-            if (!SAVED && k == L - 1 && t + gridDim.x < A.n_tiles) {
-                // the slot was consumed by the first recompute step and the next tile's stage
-                // (issued at this tile's start) has landed by now: request its P|Q rows
-                if (mbar_wait(full + (st ^ 1), (uint32_t)((j + 1) >> 1) & 1u)) gather(st ^ 1);
-            }
-            if (k == 0) {
-                // dz1 per edge (for the sender-side sum; from sG, after the barrier below) and its
-                // receiver-side segmented sum
-                constexpr int NC = H / 4;
-                float4* sS4 = reinterpret_cast<float4*>(sStage);
-                if (!SAVED) __syncthreads();   // every warp is past its last read of hb, which the staging overwrites
-#pragma unroll
-                for (int i = 0; i < CW / 4; ++i)
-                    sS4[row * NC + stage_chunk<NC>(c0 / 4 + i, row)] =
-                        make_float4(dz[4 * i], dz[4 * i + 1], dz[4 * i + 2], dz[4 * i + 3]);
-                __syncthreads();
-                {   // whole rows per warp: the tile's dz1 rows, as the MMAs read them from sG
-                    constexpr int CPR = H / 8;   // 16-byte chunks per row
-                    for (int i = tid; i < ne * CPR; i += C::NT) {
-                        const int r = i / CPR, jj = i - r * CPR;
-                        *reinterpret_cast<uint4*>(A.dz1 + ((int64_t)e0 + r) * H + 8 * jj) =
-                            *reinterpret_cast<const uint4*>(sG + tile_off(r, 8 * jj, 128, S));
-                    }
-                }
-                const int nr = r1 - r0;
-                for (int it = tid; it < nr * NC; it += C::NT) {
-                    const int rr = it / NC, c = it % NC;
-                    const int32_t b0 = sRp[rr], b1 = sRp[rr + 1];
-                    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-                    for (int32_t e = b0; e < b1; ++e) {
-                        const float4 u4 = sS4[e * NC + stage_chunk<NC>(c, e)];
-                        acc.x += u4.x;
-                        acc.y += u4.y;
-                        acc.z += u4.z;
-                        acc.w += u4.w;
-                    }
-                    *reinterpret_cast<float4*>(A.dP + (int64_t)(r0 + rr) * H + 4 * c) = acc;
-                }
-            }
-            mma_wait();
-            float dh[CW];
-            ld_acc<CW>(tWork, q, c0, dh);
-            if (k > 0) {
-                float hv[CW];
-                ld_row_tile<CW>(sHB + (k - 1) * C::TILE, row, c0, S, hv);
-                elu_bwd2<CW>(dz, dh, hv);
-            } else {
-                float o[CW];
-#pragma unroll
-                for (int i = 0; i < CW; ++i) o[i] = gv[i] + dh[i];      // residual + W1c^T dz1
-                st_row_tile<CW>(sDE, row, c0, S, o);   // copied out by whole rows after the next barrier
-            }
-            tc_fence_before();
-        }
-        first = false;
-        ok = ok && mbar_wait(bar_w, ph_w);   // the last wgrad reads this tile's e stage and sG
-        ph_w ^= 1;
-        ph_h ^= hmask;
-        __syncthreads();   // every row of de_in is in the stage's de tile
-        {
-            constexpr int CPR = H / 8;
-            for (int i = tid; i < ne * CPR; i += C::NT) {
-                const int r = i / CPR, jj = i - r * CPR;
-                *reinterpret_cast<uint4*>(A.de_in + ((int64_t)e0 + r) * H + 8 * jj) =
-                    *reinterpret_cast<const uint4*>(sDE + tile_off(r, 8 * jj, 128, S));
-            }
-        }
-        fence_proxy_async();
-        if (__syncthreads_or(!ok)) break;   // stage release; the block leaves together after a timeout
-        tc_fence_after();
-    }
-    if (p_pending) mbar_wait(p_full, ph_p);
-    if (SAVED && tid == 0)   // loads issued before a timeout ended the tile loop
-        for (int k = 0; k < L - 1; ++k)
-            if ((h_pend >> k) & 1u) mbar_wait(h_full + k, (ph_h >> k) & 1u);
-    cp_async_wait_all();
-    tc_fence_before();
-    ok = __syncthreads_and(ok) != 0;
-    tc_fence_after();
-    float* part = A.part + (int64_t)blockIdx.x * A.pstride;
-    if (ok) {
-        int64_t off = 0;
-        for (int k = 0; k < L; ++k) {
-            const int N = H + 16;
-            if (!first) flush_acc<C::CG>(tDW(k), N, H, q, lane, g, part + off);
-            else
-                for (int i = tid; i < H * N; i += C::NT) part[off + i] = 0.f;
-            off += (int64_t)H * N;
-        }
-        if constexpr (LNT) {
-            float ag[CW], ab[CW];
-#pragma unroll
-            for (int i0 = 0; i0 < CW; i0 += 16) {
-                tmem_ld16(tLN + i0, ag + i0);
-                tmem_ld16(tLN + CW + i0, ab + i0);
-            }
-            tmem_ld_wait();
-            rows_reduce_store<CW>(ag, sRed, q, lane, g, c0, part + off);
-            rows_reduce_store<CW>(ab, sRed, q, lane, g, c0, part + off + H);
-        }
-    }
-    if constexpr (!LNT) {   // after the L weight-gradient blocks [H x (H+16)]
-        const int64_t ln_off = (int64_t)L * H * (H + 16);
-        colsum_store<H, ACW>(acc_g, sRed, q, lane, c0, tid, C::NT, part + ln_off);
-        colsum_store<H, ACW>(acc_b, sRed, q, lane, c0, tid, C::NT, part + ln_off + H);
-    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1284,7 +773,7 @@ int backward_h(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
                cudaStream_t s, const __nv_bfloat16* act) {
     using C = CfgB<H>;
     const int Le = W.edge.n_lin, Ln = W.node.n_lin;
-    GNN_REQUIRE(edge_bwd_tcols<H>(Le) <= 512 && node_bwd_tcols<H>(Ln) <= 512, GNN_EUNSUPPORTED,
+    GNN_REQUIRE(edge_backward_supported(H, Le) && node_bwd_tcols<H>(Ln) <= 512, GNN_EUNSUPPORTED,
                 "gnn_mp_backward: BF16 backward at H=%d supports at most %d Linear layers per MLP", H,
                 H == 64 ? 4 : 7);
     BwdWs w = carve_bwd(ws, G, H, Le, Ln, a_star == nullptr);
@@ -1357,46 +846,20 @@ int backward_h(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
     }
     // 3. edge MLP adjoint
     if (E > 0) {
-        CUtensorMap tm_e, tm_de, tm_h;
-        if ((rc = make_row_tmap(&tm_e, e_in, E, H))) return rc;
-        if ((rc = make_row_tmap(&tm_de, de_out ? (const void*)de_out : (const void*)e_in, E, H))) return rc;
-        tm_h = tm_e;
-        if (act && (rc = make_row_tmap(&tm_h, act, (int64_t)(Le - 1) * G.n_edge_tiles * 128, H))) return rc;
-        EdgeBwdArgs A;
-        GNN_REQUIRE(G.tile_meta && ((uintptr_t)G.tile_meta & 15) == 0, GNN_EINVAL,
-                    "gnn_mp_backward: tile_meta must be a 16-byte aligned device array");
-        A.tile_meta = (const uint8_t*)G.tile_meta;
-        A.n_tiles = G.n_edge_tiles;
-        A.pq = w.pq;
-        A.q = w.pq + NR * H;
-        A.da = w.da;
-        A.has_de_out = de_out != nullptr;
-        A.de_in = de_in;
-        A.dz1 = w.dz1;
-        A.dP = w.dP;
-        A.part = w.part;
-        A.pstride = edge_pstride(H, Le);
-        A.mlp = mlp_dev(W.edge);
-        A.eps = cfg.ln_eps;
-        A.act_rows = G.n_edge_tiles * 128;
-        const EdgeBwdSmem P = edge_bwd_smem<H>(Le);
+        EdgeBackward o{};
+        o.pq = w.pq;
+        o.da = w.da;
+        o.e_in = e_in;
+        o.de_out = de_out;
+        o.act = act;
+        o.de_in = de_in;
+        o.dz1 = w.dz1;
+        o.dP = w.dP;
+        o.part = w.part;
+        o.pstride = edge_pstride(H, Le);
+        o.eps = cfg.ln_eps;
         int grid = 0;
-        const bool lnt = edge_bwd_ln_in_tmem<H>(Le);
-        auto run = [&](auto kern, uint32_t cols) -> int {
-            int r = persistent_grid(kern, C::NT, P.total, cols, G.n_edge_tiles, &grid);
-            if (r) return r;
-            grid = std::min(grid, nsm);
-            {
-                ProfScope _ps(s, "k_edge_bwd");
-                kern<<<grid, C::NT, P.total, s>>>(tm_e, tm_de, tm_h, A);
-            }
-            GNN_LAUNCH_CHECK("k_edge_bwd");
-            return GNN_OK;
-        };
-        const uint32_t cols_l = pow2_cols(edge_bwd_tcols<H>(Le) + 2 * H), cols = pow2_cols(edge_bwd_tcols<H>(Le));
-        if (act) rc = lnt ? run(k_edge_bwd<H, true, true>, cols_l) : run(k_edge_bwd<H, false, true>, cols);
-        else rc = lnt ? run(k_edge_bwd<H, true, false>, cols_l) : run(k_edge_bwd<H, false, false>, cols);
-        if (rc) return rc;
+        if ((rc = edge_backward(G, H, W, o, &grid, s))) return rc;
         RedSeg seg[MAX_SEGS];
         int n = 0;
         int64_t off = 0;
@@ -1409,7 +872,7 @@ int backward_h(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
         }
         seg[n++] = RedSeg{dW.edge.gamma, H, 1, H, off, 0};
         seg[n++] = RedSeg{dW.edge.beta, H, 1, H, off + H, 0};
-        if ((rc = reduce_grads(seg, n, w.part, A.pstride, grid, s))) return rc;
+        if ((rc = reduce_grads(seg, n, w.part, o.pstride, grid, s))) return rc;
     } else {
         GNN_CUDA_CHECK(cudaMemsetAsync(w.dP, 0, sizeof(float) * NR * H, s), "memset");
     }
