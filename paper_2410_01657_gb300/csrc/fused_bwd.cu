@@ -40,7 +40,7 @@ cudaError_t take_device_error_bwd(unsigned int* out) { return take_device_error_
 // ------------------------------------------------------------------ shared memory plans
 
 struct NodeBwdSmem {
-    uint32_t w0, w, ain, ones2, g, hb, ones, par, red, bar, tm, total;
+    uint32_t w0, w, ain, ones2, g, hb, ones, gx, par, red, bar, tm, total;
 };
 
 template <int H>
@@ -54,10 +54,11 @@ __host__ __device__ inline NodeBwdSmem node_bwd_smem(int n_lin) {
     s.g = align_up(s.ones2 + 128 * C::S2, 1024);
     s.hb = s.g + C::TILE;
     s.ones = align_up(s.hb + (n_lin - 1) * C::TILE, 1024);
-    s.par = align_up(s.ones + 128 * C::S, 16);
+    s.gx = align_up(s.ones + 128 * C::S, 1024);         // the tile's dx_out rows (FP32), then its dx_in rows
+    s.par = s.gx + 128 * H * 4;
     s.red = s.par + (n_lin + 2) * H * 4;
-    s.bar = align_up(s.red + 4 * C::CG * 128 * 4, 8);   // mma, wgrad, ready, h[GNN_MAX_LIN], xa
-    s.tm = s.bar + 8 * (4 + GNN_MAX_LIN);
+    s.bar = align_up(s.red + 4 * C::CG * 128 * 4, 8);   // mma, wgrad, ready, h[GNN_MAX_LIN], xa, gx
+    s.tm = s.bar + 8 * (5 + GNN_MAX_LIN);
     uint32_t end = s.tm + 16;
     end = end > s.g + 32768 ? end : s.g + 32768;
     s.total = end + 1024;
@@ -100,10 +101,8 @@ __host__ __device__ inline uint32_t node_bwd_tcols(int n_lin) {
 struct NodeBwdArgs {
     const float* a_star;
     const float* x;
-    const float* dx_out;
-    float* da;          // out: gradient of a* (FP32)
-    float* dx_in;       // out: dx_out + x part of the node-MLP input gradient
-    float* part;        // per-CTA weight-gradient partials
+    const float* dx_out;   // (tmap_gx; read here to prefetch)
+    float* part;           // per-CTA weight-gradient partials
     int64_t pstride;
     int64_t n_rows;
     MlpDev mlp;
@@ -116,9 +115,20 @@ struct NodeBwdArgs {
 // arrive by TMA into the activation buffers and the input tile, each refilled
 // with the next tile's rows once its last reader has passed (as in the edge adjoint),
 // and only the last Linear is recomputed; a* and x are not read.
+//
+// A tile is a chain of 8 (5) dependent MMA and epilogue steps, 512 threads with
+// 16 columns of a row each; what it moves (five FP32 rows of H per node) travels
+// as whole rows: a* and x by coalesced pieces straight into the operand tile,
+// dx_out by TMA into gx, where dx_in replaces it, and dx_in and da* (staged over
+// the dead dz and h tiles) leave by TMA stores. With per-thread row accesses the
+// loads and stores alone held the warps 15 cycles per issue (551k rows at H = 64: 0.52 ms, now
+// 0.34; at H = 32 with 7 Linears 0.39 and 0.33).
 template <int H, bool SAVED>
 __global__ void __launch_bounds__(CfgB<H>::NT, 1) k_node_bwd(const __grid_constant__ CUtensorMap tmap_h,
                                                             const __grid_constant__ CUtensorMap tmap_xa,
+                                                            const __grid_constant__ CUtensorMap tmap_gx,
+                                                            const __grid_constant__ CUtensorMap tmap_dx,
+                                                            const __grid_constant__ CUtensorMap tmap_da,
                                                             NodeBwdArgs A) {
     using C = CfgB<H>;
     extern __shared__ uint8_t smem_raw[];
@@ -138,6 +148,10 @@ __global__ void __launch_bounds__(CfgB<H>::NT, 1) k_node_bwd(const __grid_consta
     uint64_t* ready = bar + 2;                                  // one arrival per warp before an MMA
     uint64_t* h_full = bar + 3;                                 // SAVED: h_k of the tile has landed
     uint64_t* xa_full = bar + 3 + GNN_MAX_LIN;                  // SAVED: the tile's [a*, x] rows have landed
+    uint64_t* gx_full = bar + 4 + GNN_MAX_LIN;                  // the tile's dx_out rows have landed
+    uint8_t* sGX = sm + P.gx;
+    // FP32 da* rows [128 x H]: over dz and h_0; SAVED, where the next h_0 is on its way, over the input tile
+    uint8_t* sDA = SAVED ? sAin : sm + P.g;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + P.tm);
     constexpr int S = C::S, S2 = C::S2, CW = C::CW;
     const uint32_t NCOLS = pow2_cols(node_bwd_tcols<H>(L));
@@ -153,6 +167,7 @@ __global__ void __launch_bounds__(CfgB<H>::NT, 1) k_node_bwd(const __grid_consta
         mbar_init(bar, 1);
         mbar_init(bar_w, 1);
         mbar_init(ready, C::NT / 32);
+        mbar_init(gx_full, 1);
         if (SAVED) {
             for (int k = 0; k < L - 1; ++k) mbar_init(h_full + k, 1);
             mbar_init(xa_full, 1);
@@ -232,6 +247,14 @@ __global__ void __launch_bounds__(CfgB<H>::NT, 1) k_node_bwd(const __grid_consta
         for (int k = 0; k < L - 1; ++k) load_h(k, blockIdx.x);
         load_xa(blockIdx.x);
     }
+    uint32_t ph_gx = 0;
+    bool gx_pend = false;   // thread 0
+    auto load_gx = [&](int64_t tt) {
+        mbar_arrive_expect_tx(gx_full, 128 * H * 4);
+        tma_f32_tile<H>(sGX, &tmap_gx, tt * 128, gx_full);
+        gx_pend = true;
+    };
+    if (tid == 0 && (int64_t)blockIdx.x < n_tiles) load_gx(blockIdx.x);
 
     for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
         if (tid == 0 && t + gridDim.x < n_tiles) {   // the next tile's input rows into L2
@@ -241,44 +264,31 @@ __global__ void __launch_bounds__(CfgB<H>::NT, 1) k_node_bwd(const __grid_consta
             prefetch_l2(A.x + rn * H, nb);
             prefetch_l2(A.dx_out + rn * H, nb);
         }
-        const int64_t r = t * 128 + row;
-        const bool valid = r < A.n_rows;
-        float gv[CW];
-        if constexpr (SAVED) {
-            if (valid) {
-                const float4* pg = reinterpret_cast<const float4*>(A.dx_out + r * H + c0);
+        if constexpr (!SAVED) {   // the operand tile [a*, x] by pieces of four columns: consecutive threads, whole rows
+            constexpr int PPR = H / 4, IT = 128 * PPR / C::NT;
+            const int nv = (int)std::min<int64_t>(128, A.n_rows - t * 128);
+            float4 av[IT], xv[IT];
 #pragma unroll
-                for (int i = 0; i < CW / 4; ++i) {
-                    const float4 z = __ldg(pg + i);
-                    gv[4 * i] = z.x; gv[4 * i + 1] = z.y; gv[4 * i + 2] = z.z; gv[4 * i + 3] = z.w;
+            for (int i = 0; i < IT; ++i) {
+                const int p = tid + i * C::NT;
+                av[i] = xv[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (p / PPR < nv) {
+                    av[i] = __ldg(reinterpret_cast<const float4*>(A.a_star + t * 128 * H) + p);
+                    xv[i] = __ldg(reinterpret_cast<const float4*>(A.x + t * 128 * H) + p);
                 }
-            } else {
-#pragma unroll
-                for (int i = 0; i < CW; ++i) gv[i] = 0.f;
-            }
-        } else {
-            float xv[CW], av[CW];
-            if (valid) {
-                const float4* pa = reinterpret_cast<const float4*>(A.a_star + r * H + c0);
-                const float4* px = reinterpret_cast<const float4*>(A.x + r * H + c0);
-                const float4* pg = reinterpret_cast<const float4*>(A.dx_out + r * H + c0);
-#pragma unroll
-                for (int i = 0; i < CW / 4; ++i) {
-                    float4 u = __ldg(pa + i), w = __ldg(px + i), z = __ldg(pg + i);
-                    av[4 * i] = u.x; av[4 * i + 1] = u.y; av[4 * i + 2] = u.z; av[4 * i + 3] = u.w;
-                    xv[4 * i] = w.x; xv[4 * i + 1] = w.y; xv[4 * i + 2] = w.z; xv[4 * i + 3] = w.w;
-                    gv[4 * i] = z.x; gv[4 * i + 1] = z.y; gv[4 * i + 2] = z.z; gv[4 * i + 3] = z.w;
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < CW; ++i) av[i] = xv[i] = gv[i] = 0.f;
             }
 #pragma unroll
-            for (int i = 0; i < CW; i += 8) {
-                st_tile8(sAin, row, c0 + i, 128, S2, av + i);
-                st_tile8(sAin, row, H + c0 + i, 128, S2, xv + i);
+            for (int i = 0; i < IT; ++i) {
+                const int p = tid + i * C::NT, rr = p / PPR, c = 4 * (p % PPR);
+                *reinterpret_cast<uint2*>(sAin + tile_off(rr, c, 128, S2)) =
+                    make_uint2(pack_bf16x2(av[i].x, av[i].y), pack_bf16x2(av[i].z, av[i].w));
+                *reinterpret_cast<uint2*>(sAin + tile_off(rr, H + c, 128, S2)) =
+                    make_uint2(pack_bf16x2(xv[i].x, xv[i].y), pack_bf16x2(xv[i].z, xv[i].w));
             }
         }
+        // (thread 0 issues the tile's first MMA after the previous tile's da* store has read the dz and h
+        // tiles: nobody writes those before that MMA has completed)
+        if (tid == 0) bulk_wait_read_all();
         // ---- recompute the chain (SAVED: only the last Linear, from the saved h_{L-2})
         float v[CW];
         if constexpr (SAVED) {
@@ -310,6 +320,18 @@ __global__ void __launch_bounds__(CfgB<H>::NT, 1) k_node_bwd(const __grid_consta
             }
         }
         tc_fence_before();
+        float gv[CW];   // dx_out (zero past n_rows)
+        ok = ok && mbar_wait(gx_full, ph_gx);
+        ph_gx ^= 1;
+        __syncwarp();
+        auto load_gv = [&] {
+#pragma unroll
+            for (int i = 0; i < CW / 4; ++i) {
+                const float4 z = ld_f32x4_tile<H>(sGX, row, c0 + 4 * i);
+                gv[4 * i] = z.x; gv[4 * i + 1] = z.y; gv[4 * i + 2] = z.z; gv[4 * i + 3] = z.w;
+            }
+        };
+        load_gv();
         // ---- LayerNorm adjoint (statistics and adjoint sums in one exchange)
         float dz[CW];
 #pragma unroll
@@ -362,26 +384,43 @@ __global__ void __launch_bounds__(CfgB<H>::NT, 1) k_node_bwd(const __grid_consta
                 float da[CW], dxp[CW];
                 ld_acc<CW>(tWork, q, c0, da);
                 ld_acc<CW>(tWork, q, H + c0, dxp);
-                if (valid) {
-                    float4* pda = reinterpret_cast<float4*>(A.da + r * H + c0);
-                    float4* pdx = reinterpret_cast<float4*>(A.dx_in + r * H + c0);
+                ok = ok && mbar_wait(bar_w, ph_w);   // dz and h are dead
 #pragma unroll
-                    for (int i = 0; i < CW / 4; ++i) {
-                        pda[i] = make_float4(da[4 * i], da[4 * i + 1], da[4 * i + 2], da[4 * i + 3]);
-                        pdx[i] = make_float4(gv[4 * i] + dxp[4 * i], gv[4 * i + 1] + dxp[4 * i + 1],
-                                             gv[4 * i + 2] + dxp[4 * i + 2], gv[4 * i + 3] + dxp[4 * i + 3]);
-                    }
+                for (int i = 0; i < CW / 4; ++i) {
+                    st_f32x4_tile<H>(sDA, row, c0 + 4 * i, make_float4(da[4 * i], da[4 * i + 1], da[4 * i + 2], da[4 * i + 3]));
+                    st_f32x4_tile<H>(sGX, row, c0 + 4 * i,
+                                     make_float4(gv[4 * i] + dxp[4 * i], gv[4 * i + 1] + dxp[4 * i + 1],
+                                                 gv[4 * i + 2] + dxp[4 * i + 2], gv[4 * i + 3] + dxp[4 * i + 3]));
                 }
+                fence_proxy_async();
             }
             tc_fence_before();
         }
         first = false;
-        ok = ok && mbar_wait(bar_w, ph_w);   // the last wgrad reads sAin and sG
         ph_w ^= 1;
         ph_h ^= hmask;
-        if (SAVED && tid == 0 && ok && t + gridDim.x < n_tiles) load_xa(t + gridDim.x);   // sAin is free
+        if (tid == 0) gx_pend = false;
+        __syncwarp();
         if (__syncthreads_or(!ok)) break;   // the block leaves together after a timeout
         tc_fence_after();
+        if (tid == 0) {   // da* and dx_in leave; the next tile's rows come once they have been read
+            constexpr int BW = H < 32 ? H : 32;
+#pragma unroll
+            for (int b = 0; b < H / BW; ++b) {
+                tma_store_2d(&tmap_dx, b * BW, (int32_t)(t * 128), sGX + b * 128 * BW * 4);
+                tma_store_2d(&tmap_da, b * BW, (int32_t)(t * 128), sDA + b * 128 * BW * 4);
+            }
+            bulk_commit();
+            if (t + gridDim.x < n_tiles) {
+                bulk_wait_read_all();
+                load_gx(t + gridDim.x);
+                if (SAVED) load_xa(t + gridDim.x);
+            }
+        }
+    }
+    if (tid == 0) {
+        if (gx_pend) mbar_wait(gx_full, ph_gx);
+        bulk_wait_all();
     }
     if (SAVED && tid == 0) {   // loads issued before a timeout ended the tile loop
         for (int k = 0; k < L - 1; ++k)
@@ -796,8 +835,6 @@ int backward_h(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
         A.a_star = astar;
         A.x = x_in;
         A.dx_out = dx_out;
-        A.da = w.da;
-        A.dx_in = dx_in;
         A.part = w.part;
         A.pstride = node_pstride(H, Ln);
         A.n_rows = NR;
@@ -805,9 +842,12 @@ int backward_h(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
         A.eps = cfg.ln_eps;
         A.act_rows = (NR + 127) / 128 * 128;
         const NodeBwdSmem P = node_bwd_smem<H>(Ln);
-        CUtensorMap tm_hn, tm_xa;
+        CUtensorMap tm_hn, tm_xa, tm_gx, tm_dx, tm_da;
         std::memset(&tm_hn, 0, sizeof(tm_hn));
         std::memset(&tm_xa, 0, sizeof(tm_xa));
+        if ((rc = make_f32_tmap(&tm_gx, dx_out, NR, H))) return rc;
+        if ((rc = make_f32_tmap(&tm_dx, dx_in, NR, H))) return rc;
+        if ((rc = make_f32_tmap(&tm_da, w.da, NR, H))) return rc;
         if (act) {
             const __nv_bfloat16* an = act + mp_act_elems_edge(G, W, H);
             if ((rc = make_row_tmap(&tm_hn, an, (int64_t)(Ln - 1) * A.act_rows, H))) return rc;
@@ -820,7 +860,7 @@ int backward_h(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
             grid = std::min(grid, nsm);
             {
                 ProfScope _ps(s, "k_node_bwd");
-                kern<<<grid, C::NT, P.total, s>>>(tm_hn, tm_xa, A);
+                kern<<<grid, C::NT, P.total, s>>>(tm_hn, tm_xa, tm_gx, tm_dx, tm_da, A);
             }
             GNN_LAUNCH_CHECK("k_node_bwd");
             return GNN_OK;
