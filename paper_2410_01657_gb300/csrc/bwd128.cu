@@ -1549,7 +1549,7 @@ int backward_h128(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp
         GNN_CUDA_CHECK(cudaMemsetAsync(w.dP, 0, sizeof(float) * NR * H, s), "memset");
     }
     // 4. projection adjoint: sender-side sums, dx_in += [dP dQ] [W1a; W1b], dW1a, dW1b
-    return proj_backward(G, H, W, x_in, w.dP, w.dz1, w.pq, dx_in, dW, w.part, s);   // (P|Q is done with)
+    return proj_backward128(G, W, x_in, w.dP, w.dz1, w.pq, dx_in, dW, w.part, s);   // (P|Q is done with)
 }
 
 }  // namespace fused

@@ -110,11 +110,11 @@ bool edge_backward_supported(int H, int n_lin);
 int edge_backward(const gnn_graph_dev& G, int H, const gnn_mp_params& W, const EdgeBackward& o, int* grid,
                   cudaStream_t s);
 
-// Projection adjoint of the BF16 backward: dQ (scratch, [n_rows x H]) from dz1 over each row's sent
+// Projection adjoint of the BF16 backward at H = 128: dQ (scratch, [n_rows x H]) from dz1 over each row's sent
 // edges, dx_in += dP W1a + dQ W1b, dW1a and dW1b added into dW.edge.W[0].
-int proj_backward(const gnn_graph_dev& G, int H, const gnn_mp_params& W, const float* x_in, const float* dP,
-                  const __nv_bfloat16* dz1, __nv_bfloat16* dQ, float* dx_in, const gnn_mp_params& dW, float* part,
-                  cudaStream_t s);
+int proj_backward128(const gnn_graph_dev& G, const gnn_mp_params& W, const float* x_in, const float* dP,
+                     const __nv_bfloat16* dz1, __nv_bfloat16* dQ, float* dx_in, const gnn_mp_params& dW, float* part,
+                     cudaStream_t s);
 
 // Layered BF16 backward at H = 128 (recomputation, per-Linear adjoint kernels).
 size_t backward_h128_ws(const gnn_graph_dev& G, const gnn_mp_params& W);

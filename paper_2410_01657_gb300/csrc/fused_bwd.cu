@@ -668,62 +668,76 @@ __global__ void __launch_bounds__(CfgP<H>::NT, H >= 128 ? 1 : 2) k_proj_bwd(Proj
 
 // ------------------------------------------------------------------ partial reduction
 
-// dst[r*dst_ld + c] += sum over CTAs b (ascending) of part[b*pstride + src_off + r*src_ld + c]
+// dst[r*dst_ld + c] += sum over CTAs b of part[b*pstride + src_off + r*src_ld + c]. A block
+// takes 32 elements; its eight warps take every eighth CTA, in order, eight loads
+// in flight each, and their sums are added in warp order: the sum over 152 CTAs
+// is three round trips to L2 where one thread per element made ten (8 us a
+// launch at 0.1 to 12 MB of partials; 3 now).
 struct RedArgs {
     RedSeg seg[MAX_SEGS];
     int n_seg;
-    int64_t seg_start[MAX_SEGS + 1];   // prefix sums of rows*cols
-    const float* part;
-    int64_t pstride;
-    int n_cta;
+    int blk[MAX_SEGS + 1];   // first block of each segment
 };
 
-__global__ void k_reduce_grads(RedArgs A) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= A.seg_start[A.n_seg]) return;
+__global__ void __launch_bounds__(256) k_reduce_grads(const __grid_constant__ RedArgs A) {
+    __shared__ float red[8][32];
     int s = 0;
-    while (i >= A.seg_start[s + 1]) ++s;
+    while ((int)blockIdx.x >= A.blk[s + 1]) ++s;
     const RedSeg& sg = A.seg[s];
-    const int64_t j = i - A.seg_start[s];
-    const int r = (int)(j / sg.cols), c = (int)(j % sg.cols);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int j = ((int)blockIdx.x - A.blk[s]) * 32 + lane;
+    const int r = j / sg.cols, c = j % sg.cols;
+    const bool in = r < sg.rows;
     float acc = 0.f;
-    const float* p = A.part + sg.src_off + (int64_t)r * sg.src_ld + c;
-    // CTA partials in ascending order; the loads of 16 CTAs are requested together
-    // (the sum is one latency-bound pass over a few tens of MB)
-    constexpr int U = 16;
-    int b = 0;
-    for (; b + U <= A.n_cta; b += U) {
-        float v[U];
+    if (in) {
+        const float* p = sg.part + sg.src_off + (int64_t)r * sg.src_ld + c;
+        constexpr int U = 8;
+        for (int b0 = w; b0 < sg.n_cta; b0 += 8 * U) {
+            float v[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) v[u] = __ldg(p + (int64_t)(b + u) * A.pstride);
+            for (int u = 0; u < U; ++u) v[u] = b0 + 8 * u < sg.n_cta ? __ldg(p + (int64_t)(b0 + 8 * u) * sg.pstride) : 0.f;
 #pragma unroll
-        for (int u = 0; u < U; ++u) acc += v[u];
+            for (int u = 0; u < U; ++u) acc += v[u];
+        }
     }
-    for (; b < A.n_cta; ++b) acc += __ldg(p + (int64_t)b * A.pstride);
-    sg.dst[(int64_t)r * sg.dst_ld + c] += acc;
+    red[w][lane] = acc;
+    __syncthreads();
+    if (w == 0 && in) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t += red[k][lane];
+        sg.dst[(int64_t)r * sg.dst_ld + c] += t;
+    }
 }
 
 // =================================================================== host side
 
-int reduce_grads(RedSeg* segs, int n, const float* part, int64_t pstride, int n_cta, cudaStream_t s) {
+int reduce_grads(RedSeg* segs, int n, cudaStream_t s) {
     RedArgs A{};
-    A.n_seg = n;
-    A.seg_start[0] = 0;
+    GNN_REQUIRE(n <= MAX_SEGS, GNN_EUNSUPPORTED, "reduce_grads: too many segments");
     for (int i = 0; i < n; ++i) {
-        A.seg[i] = segs[i];
-        A.seg_start[i + 1] = A.seg_start[i] + (int64_t)segs[i].rows * segs[i].cols;
+        if (segs[i].n_cta <= 0) continue;
+        A.seg[A.n_seg] = segs[i];
+        A.blk[A.n_seg + 1] = A.blk[A.n_seg] + (segs[i].rows * segs[i].cols + 31) / 32;
+        ++A.n_seg;
     }
-    A.part = part;
-    A.pstride = pstride;
-    A.n_cta = n_cta;
-    const int64_t tot = A.seg_start[n];
-    if (tot == 0) return GNN_OK;
+    const int blocks = A.blk[A.n_seg];
+    if (blocks == 0) return GNN_OK;
     {
         ProfScope _ps(s, "k_reduce_grads");
-        k_reduce_grads<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(A);
+        k_reduce_grads<<<blocks, 256, 0, s>>>(A);
     }
     GNN_LAUNCH_CHECK("k_reduce_grads");
     return GNN_OK;
+}
+
+int reduce_grads(RedSeg* segs, int n, const float* part, int64_t pstride, int n_cta, cudaStream_t s) {
+    for (int i = 0; i < n; ++i) {
+        segs[i].part = part;
+        segs[i].pstride = pstride;
+        segs[i].n_cta = n_cta;
+    }
+    return reduce_grads(segs, n, s);
 }
 
 namespace {
@@ -736,7 +750,7 @@ struct BwdWs {
     float* da;
     float* dP;
     __nv_bfloat16* dz1;
-    float* part;
+    float *part_node, *part_edge, *part_proj;
     size_t bytes;
 };
 
@@ -760,10 +774,11 @@ BwdWs carve_bwd(void* ws, const gnn_graph_dev& G, int H, int Le, int Ln, bool ne
     w.da = (float*)take((size_t)NR * H * 4);
     w.dP = (float*)take((size_t)NR * H * 4);
     w.dz1 = (__nv_bfloat16*)take((size_t)E * H * 2);
-    // per-CTA weight-gradient partials: one CTA per SM for the edge and node kernels,
-    // up to two per SM for the projection kernel
-    const int64_t ps = std::max(edge_pstride(H, Le), node_pstride(H, Ln));
-    w.part = (float*)take((size_t)std::max(ncta * ps, 2 * ncta * proj_pstride(H)) * 4);
+    // per-CTA weight-gradient partials: one CTA per SM for the edge and node kernels, up to two per
+    // SM for the projection kernel; apart, so that one launch sums them all
+    w.part_node = (float*)take((size_t)ncta * node_pstride(H, Ln) * 4);
+    w.part_edge = (float*)take((size_t)ncta * edge_pstride(H, Le) * 4);
+    w.part_proj = (float*)take((size_t)2 * ncta * proj_pstride(H) * 4);
     w.bytes = off + 256;
     return w;
 }
@@ -771,7 +786,8 @@ BwdWs carve_bwd(void* ws, const gnn_graph_dev& G, int H, int Le, int Ln, bool ne
 template <int H>
 int proj_backward_h(const gnn_graph_dev& G, const gnn_mp_params& W, const float* x_in, const float* dP,
                     const __nv_bfloat16* dz1, __nv_bfloat16* dQ, float* dx_in, const gnn_mp_params& dW, float* part,
-                    cudaStream_t s) {
+                    RedSeg* seg, int* n_seg, cudaStream_t s) {
+    *n_seg = 0;
     const int64_t NR = G.n_rows;
     if (NR == 0) return GNN_OK;
     ProjBwdArgs A;
@@ -799,10 +815,10 @@ int proj_backward_h(const gnn_graph_dev& G, const gnn_mp_params& W, const float*
         k_proj_bwd<H><<<grid, CfgP<H>::NT, P.total, s>>>(A);
     }
     GNN_LAUNCH_CHECK("k_proj_bwd");
-    RedSeg seg[2];
-    seg[0] = RedSeg{dW.edge.W[0], 3 * H, H, H, 0, H};                     // dW1a -> W1[:, 0:H]
-    seg[1] = RedSeg{dW.edge.W[0] + H, 3 * H, H, H, (int64_t)H * H, H};    // dW1b -> W1[:, H:2H]
-    return reduce_grads(seg, 2, part, A.pstride, grid, s);
+    seg[0] = RedSeg{dW.edge.W[0], 3 * H, H, H, 0, H, part, A.pstride, grid};                     // dW1a -> W1[:, 0:H]
+    seg[1] = RedSeg{dW.edge.W[0] + H, 3 * H, H, H, (int64_t)H * H, H, part, A.pstride, grid};    // dW1b -> W1[:, H:2H]
+    *n_seg = 2;
+    return GNN_OK;
 }
 
 template <int H>
@@ -829,13 +845,15 @@ int backward_h(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
     }
     const float* astar = a_star ? a_star : w.a;
     const int nsm = num_sms();
+    RedSeg seg[MAX_SEGS];
+    int n = 0;
     // 1. node MLP adjoint
     {
         NodeBwdArgs A;
         A.a_star = astar;
         A.x = x_in;
         A.dx_out = dx_out;
-        A.part = w.part;
+        A.part = w.part_node;
         A.pstride = node_pstride(H, Ln);
         A.n_rows = NR;
         A.mlp = mlp_dev(W.node);
@@ -866,19 +884,19 @@ int backward_h(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
             return GNN_OK;
         };
         if ((rc = act ? run(k_node_bwd<H, true>) : run(k_node_bwd<H, false>))) return rc;
-        RedSeg seg[MAX_SEGS];
-        int n = 0;
         int64_t off = 0;
+        auto add = [&](float* dst, int ld, int rows, int cols, int64_t src, int64_t src_ld) {
+            seg[n++] = RedSeg{dst, ld, rows, cols, src, src_ld, A.part, A.pstride, grid};
+        };
         for (int k = 0; k < Ln; ++k) {
             const int in = k == 0 ? 2 * H : H;
             const int N = in + 16;
-            seg[n++] = RedSeg{dW.node.W[k], in, H, in, off, N};
-            seg[n++] = RedSeg{dW.node.b[k], 1, H, 1, off + in, N};
+            add(dW.node.W[k], in, H, in, off, N);
+            add(dW.node.b[k], 1, H, 1, off + in, N);
             off += (int64_t)H * N;
         }
-        seg[n++] = RedSeg{dW.node.gamma, H, 1, H, off, 0};
-        seg[n++] = RedSeg{dW.node.beta, H, 1, H, off + H, 0};
-        if ((rc = reduce_grads(seg, n, w.part, A.pstride, grid, s))) return rc;
+        add(dW.node.gamma, H, 1, H, off, 0);
+        add(dW.node.beta, H, 1, H, off + H, 0);
     }
     // 2. adjoint of the halo swap + sync
     if (cfg.halo_mode == GNN_HALO_SYNC) {
@@ -895,29 +913,32 @@ int backward_h(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
         o.de_in = de_in;
         o.dz1 = w.dz1;
         o.dP = w.dP;
-        o.part = w.part;
+        o.part = w.part_edge;
         o.pstride = edge_pstride(H, Le);
         o.eps = cfg.ln_eps;
         int grid = 0;
         if ((rc = edge_backward(G, H, W, o, &grid, s))) return rc;
-        RedSeg seg[MAX_SEGS];
-        int n = 0;
         int64_t off = 0;
+        auto add = [&](float* dst, int ld, int rows, int cols, int64_t src, int64_t src_ld) {
+            seg[n++] = RedSeg{dst, ld, rows, cols, src, src_ld, o.part, o.pstride, grid};
+        };
         for (int k = 0; k < Le; ++k) {
             const int N = H + 16;
-            if (k == 0) seg[n++] = RedSeg{dW.edge.W[0] + 2 * H, 3 * H, H, H, off, N};   // W1c columns of W1
-            else seg[n++] = RedSeg{dW.edge.W[k], H, H, H, off, N};
-            seg[n++] = RedSeg{dW.edge.b[k], 1, H, 1, off + H, N};
+            if (k == 0) add(dW.edge.W[0] + 2 * H, 3 * H, H, H, off, N);   // W1c columns of W1
+            else add(dW.edge.W[k], H, H, H, off, N);
+            add(dW.edge.b[k], 1, H, 1, off + H, N);
             off += (int64_t)H * N;
         }
-        seg[n++] = RedSeg{dW.edge.gamma, H, 1, H, off, 0};
-        seg[n++] = RedSeg{dW.edge.beta, H, 1, H, off + H, 0};
-        if ((rc = reduce_grads(seg, n, w.part, o.pstride, grid, s))) return rc;
+        add(dW.edge.gamma, H, 1, H, off, 0);
+        add(dW.edge.beta, H, 1, H, off + H, 0);
     } else {
         GNN_CUDA_CHECK(cudaMemsetAsync(w.dP, 0, sizeof(float) * NR * H, s), "memset");
     }
     // 4. projection adjoint: sender-side sums, dx_in += [dP dQ] [W1a; W1b], dW1a, dW1b
-    return proj_backward_h<H>(G, W, x_in, w.dP, w.dz1, w.pq, dx_in, dW, w.part, s);   // (P|Q is done with)
+    // (P|Q is done with)
+    int np = 0;
+    if ((rc = proj_backward_h<H>(G, W, x_in, w.dP, w.dz1, w.pq, dx_in, dW, w.part_proj, seg + n, &np, s))) return rc;
+    return reduce_grads(seg, n + np, s);
 }
 
 }  // namespace
@@ -927,16 +948,13 @@ size_t mp_backward_ws(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gn
     return carve_bwd(nullptr, G, cfg.hidden, W.edge.n_lin, W.node.n_lin, true).bytes;
 }
 
-int proj_backward(const gnn_graph_dev& G, int H, const gnn_mp_params& W, const float* x_in, const float* dP,
-                  const __nv_bfloat16* dz1, __nv_bfloat16* dQ, float* dx_in, const gnn_mp_params& dW, float* part,
-                  cudaStream_t s) {
-    switch (H) {
-        case 16: return proj_backward_h<16>(G, W, x_in, dP, dz1, dQ, dx_in, dW, part, s);
-        case 32: return proj_backward_h<32>(G, W, x_in, dP, dz1, dQ, dx_in, dW, part, s);
-        case 64: return proj_backward_h<64>(G, W, x_in, dP, dz1, dQ, dx_in, dW, part, s);
-        case 128: return proj_backward_h<128>(G, W, x_in, dP, dz1, dQ, dx_in, dW, part, s);
-        default: return set_error(GNN_EUNSUPPORTED, "proj_backward: H=%d", H);
-    }
+int proj_backward128(const gnn_graph_dev& G, const gnn_mp_params& W, const float* x_in, const float* dP,
+                     const __nv_bfloat16* dz1, __nv_bfloat16* dQ, float* dx_in, const gnn_mp_params& dW, float* part,
+                     cudaStream_t s) {
+    RedSeg seg[2];
+    int n = 0;
+    int rc = proj_backward_h<128>(G, W, x_in, dP, dz1, dQ, dx_in, dW, part, seg, &n, s);
+    return rc ? rc : reduce_grads(seg, n, s);
 }
 
 int mp_backward(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_params& W, const float* x_in,

@@ -163,10 +163,15 @@ struct RedSeg {
     float* dst;
     int dst_ld, rows, cols;
     int64_t src_off, src_ld;
+    const float* part;      // of n_cta CTAs, pstride apart
+    int64_t pstride;
+    int n_cta;
 };
 
-constexpr int MAX_SEGS = 2 * GNN_MAX_LIN + 4;
+constexpr int MAX_SEGS = 4 * GNN_MAX_LIN + 6;   // a layer: both MLPs' Linears, LayerNorms and the projection
 
+int reduce_grads(RedSeg* segs, int n, cudaStream_t s);
+// The same with one set of partials for all segments.
 int reduce_grads(RedSeg* segs, int n, const float* part, int64_t pstride, int n_cta, cudaStream_t s);
 
 }  // namespace fused
