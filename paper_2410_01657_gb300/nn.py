@@ -48,6 +48,15 @@ def n_mlp_tensors(dims, has_ln: bool) -> int:
     return 2 * (len(dims) - 1) + (2 if has_ln else 0)
 
 
+def zero_grads(tensors) -> tuple:
+    """(flat, views): zeroed gradient buffers shaped like ``tensors``, pieces of one
+    flat allocation, so that zeroing them is one launch instead of one per tensor
+    (a layer has 20 and more: on small graphs those launches took longer than
+    the layer's kernels)."""
+    flat = torch.zeros(sum(t.numel() for t in tensors), dtype=torch.float32, device=tensors[0].device)
+    return flat, [v.view(t.shape) for v, t in zip(flat.split([t.numel() for t in tensors]), tensors)]
+
+
 def mp_config(hidden: int, precision: str, halo: bool = True, ln_eps: float = 1e-5, flags: int = 0):
     c = B.gnn_mp_config()
     c.hidden = int(hidden)
@@ -150,7 +159,7 @@ class ConsistentMPFunction(torch.autograd.Function):
         G = ctx.G
         cfg = mp_config(*ctx.cfg_args)
         W = mp_params(*ctx.dims, params)
-        dparams = [torch.zeros_like(p) for p in params]
+        _, dparams = zero_grads(params)
         dW = mp_params(*ctx.dims, dparams)
         _, bwd = mp_workspace_sizes(G, cfg, W)
         dx = torch.empty_like(x)
@@ -213,7 +222,7 @@ class RowMLPFunction(torch.autograd.Function):
         X, *params = ctx.saved_tensors
         dims, has_ln, out_bf16, ln_eps, need_dx, bwd, sfx = ctx.meta
         P = mlp_struct(dims, params, has_ln)
-        dparams = [torch.zeros_like(p) for p in params]
+        _, dparams = zero_grads(params)
         dP = mlp_struct(dims, dparams, has_ln)
         dY = dY.to(torch.bfloat16 if out_bf16 else torch.float32).contiguous()
         dX = torch.empty_like(X) if need_dx else None
@@ -318,11 +327,13 @@ class LayerStack:
         dev = x0.device
         edt = torch.bfloat16 if precision == "bf16" else torch.float32
         self.W, self.dW, self.dparams = [], [], []
+        if not inference:   # every layer's gradients in one allocation (zero_grad is one launch)
+            self._grads, views = zero_grads([t for (te, tn, _, _) in layers for t in (*te, *tn)])
         for (te, tn, de, dn) in layers:
             tens = list(te) + list(tn)
             self.W.append(mp_params(de, dn, tens))
             if not inference:
-                dp = [torch.zeros_like(t) for t in tens]
+                dp, views = views[:len(tens)], views[len(tens):]
                 self.dparams.append(dp)
                 self.dW.append(mp_params(de, dn, dp))
         self._keep = [layers]
@@ -367,9 +378,8 @@ class LayerStack:
         return self._io(self.M - 1)[2]
 
     def zero_grad(self):
-        for dp in self.dparams:
-            for t in dp:
-                t.zero_()
+        if self.dparams:
+            self._grads.zero_()
 
     def forward(self):
         if self._act_tiles != int(self.G.struct.n_edge_tiles):
