@@ -876,6 +876,321 @@ __global__ void __launch_bounds__(kWThreads, 1) k_wgrad3(const __grid_constant__
     if (warp == 0) tmem_dealloc(tmem, NCOLS);
 }
 
+// ------------------------------------------------------------------ k_chain3
+
+// One Linear of the adjoint chain at widths <= 64, both halves in one pass over
+// dz [rows x N] and h [rows x K]: dz' = (dz W) ELU'(h) and dW += dz^T h,
+// db += column sums of dz. dz is split once for both products (its row tile is
+// the K-major operand of the first and the MN-major one of the second), h once,
+// and each row is read once instead of twice (three tensors moved instead of
+// five). Two stages of dz and one of h fill shared memory beside W; the widths
+// above 64 need twice that and keep the two launches. 3.23M edge rows at width
+// 64: 0.84 ms as it stands against 0.49 + 0.48 for the two launches: the four
+// producer warps split both operands and set the pace (HBM alone: 0.37).
+struct CArgs {
+    int64_t rows;
+    int n_tiles;
+    const float* G;      // dz [rows x N]
+    const float* H;      // h [rows x K]
+    const float* W;      // [N x K]
+    float* out;          // dz' [rows x K]
+    int N, K, db, vec;
+    float* part;         // per CTA: dW [N x K], then db [N]
+};
+
+struct CSmem {
+    uint32_t w, g, h, stg, red, bar, tm, total, wterm, gterm, hterm;
+};
+
+template <int NW, int KW>
+__host__ __device__ constexpr CSmem chain_smem() {
+    CSmem s{};
+    s.wterm = KW * NW * 2;
+    s.gterm = 128 * NW * 2;
+    s.hterm = 128 * KW * 2;
+    s.w = 0;
+    s.g = align_up(3 * s.wterm, 1024);
+    s.h = s.g + 2 * 3 * s.gterm;
+    // M = 128 views of a narrower dz tile read 32 KB from a term's start: the h stage and what follows
+    uint32_t end = s.h + 3 * s.hterm;
+    const uint32_t view = s.h - s.gterm + 32768;
+    end = end > view ? end : view;
+    s.stg = align_up(end, 16);
+    s.red = s.stg + kEpilogueWarps * kStageBytes;        // db: [128 threads][8]
+    s.bar = align_up(s.red + kProducers * 8 * 4, 8);     // full_g[2], empty_g[2], full_h, empty_h, acc_full[2], acc_empty[2], w_full[2], w_empty[2]
+    s.tm = s.bar + 14 * 8;
+    s.total = s.tm + 16 + 1024;
+    return s;
+}
+
+// Load, split and write the [128 x W] rows of one operand tile; cs: column sums (or NULL).
+template <int W, bool VEC, bool SUM>
+__device__ __forceinline__ void chain_fill(const float* src, int64_t ld, int cols, int left, uint8_t* dst, int tid,
+                                           float* cs, uint64_t* empty, bool wait, uint32_t parity, int lane, bool& ok) {
+    constexpr int U = W / 8, RS = kProducers / U, IT = 128 / RS, B = IT < 8 ? IT : 8, S = span_of(W);
+    static_assert((RS * S) % 1024 == 0, "the swizzle repeats every RS rows");
+    const int c = (tid % U) * 8, row0 = tid / U;
+    uint8_t* d0 = dst + tile_off(row0, c, 128, S);
+    const float* p = src + (int64_t)row0 * ld + c;
+    const int64_t step = RS * ld;
+#pragma unroll
+    for (int i0 = 0; i0 < IT; i0 += B) {
+        float v[B][8];
+        if (left == 128 && cols == W) {
+#pragma unroll
+            for (int i = 0; i < B; ++i) load8<VEC>(p + (i0 + i) * step, 8, v[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < B; ++i) load8<VEC>(p + (i0 + i) * step, row0 + (i0 + i) * RS < left ? cols - c : 0, v[i]);
+        }
+        if (i0 == 0 && wait) {
+            ok = warp_wait(empty, parity, lane);
+            if (!ok) return;
+        }
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            if constexpr (SUM) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) cs[k] += v[i][k];
+            }
+            uint4 h, m, l;
+            split8(v[i], h, m, l);
+            uint8_t* q = d0 + (i0 + i) * RS * S;
+            *reinterpret_cast<uint4*>(q) = h;
+            *reinterpret_cast<uint4*>(q + 128 * S) = m;
+            *reinterpret_cast<uint4*>(q + 2 * 128 * S) = l;
+        }
+    }
+    fence_proxy_async();
+    __syncwarp();
+}
+
+// NW, KW: N and K rounded up to 16, 32 or 64.
+template <int NW, int KW, bool VEC>
+__global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ CArgs A) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* sm = aligned_smem(smem_raw);
+    constexpr CSmem P = chain_smem<NW, KW>();
+    constexpr int Sg = span_of(NW), Sh = span_of(KW);
+    uint64_t* full_g = reinterpret_cast<uint64_t*>(sm + P.bar);
+    uint64_t* empty_g = full_g + 2;
+    uint64_t* full_h = full_g + 4;
+    uint64_t* empty_h = full_g + 5;
+    uint64_t* acc_full = full_g + 6;
+    uint64_t* acc_empty = full_g + 8;
+    uint64_t* w_full = full_g + 10;
+    uint64_t* w_empty = full_g + 12;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + P.tm);
+    float* sRed = reinterpret_cast<float*>(sm + P.red);
+    // TMEM: dz' of two tiles (hi hi | small products), dW of two tiles
+    constexpr uint32_t NCOLS = 6 * KW <= 128 ? 128 : (6 * KW <= 256 ? 256 : 512), WCOL = 4 * KW;
+    constexpr int CW = KW >= 32 ? KW / 2 : 16;   // dW columns per epilogue thread
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, N = A.N, K = A.K;
+
+    if (warp == 0) {
+        tmem_alloc(tslot, NCOLS);
+        tmem_relinquish();
+    }
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(full_g + i, kProducerWarps);
+            mbar_init(empty_g + i, 1);
+            mbar_init(acc_full + i, 1);
+            mbar_init(acc_empty + i, 4);
+            mbar_init(w_full + i, 1);
+            mbar_init(w_empty + i, kEpilogueWarps);
+        }
+        mbar_init(full_h, kProducerWarps);
+        mbar_init(empty_h, 1);
+        fence_mbar_init();
+    }
+    // W^T as the [KW x NW] K-major operand of dz W: row k, column n
+    for (int i = tid; i < KW * (NW / 8); i += kThreads) {
+        const int k = i / (NW / 8), n8 = (i % (NW / 8)) * 8;
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = (k < K && n8 + j < N) ? __ldg(A.W + (int64_t)(n8 + j) * K + k) : 0.f;
+        uint4 t[3];
+        split8(v, t[0], t[1], t[2]);
+        const uint32_t off = tile_off(k, n8, KW, Sg);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) *reinterpret_cast<uint4*>(sm + P.w + j * P.wterm + off) = t[j];
+    }
+    fence_proxy_async();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot;
+    float* part = A.part + (int64_t)blockIdx.x * (N * K + (A.db ? N : 0));
+
+    if (warp < kProducerWarps) {
+        float cs[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) cs[i] = 0.f;
+        bool ok = true;
+        int j = 0;
+        for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++j) {
+            if (VEC && tid == 0 && t + (int)gridDim.x < A.n_tiles) {   // the next tile's rows into L2
+                const int64_t rn = (int64_t)(t + (int)gridDim.x) * 128, nr = std::min<int64_t>(128, A.rows - rn);
+                prefetch_l2(A.G + rn * N, (uint32_t)(nr * N * 4));
+                prefetch_l2(A.H + rn * K, (uint32_t)(nr * K * 4));
+            }
+            const int64_t r0 = (int64_t)t * 128;
+            const int left = (int)std::min<int64_t>(128, A.rows - r0), st = j & 1;
+            chain_fill<NW, VEC, true>(A.G + r0 * N, N, N, left, sm + P.g + st * 3 * P.gterm, tid, cs, empty_g + st, j >= 2,
+                                      (uint32_t)((j >> 1) - 1) & 1u, lane, ok);
+            if (!ok) break;
+            if (lane == 0) mbar_arrive(full_g + st);
+            chain_fill<KW, VEC, false>(A.H + r0 * K, K, K, left, sm + P.h, tid, nullptr, empty_h, j >= 1,
+                                       (uint32_t)(j - 1) & 1u, lane, ok);
+            if (!ok) break;
+            if (lane == 0) mbar_arrive(full_h);
+        }
+        if (A.db) {   // column sums of dz: threads of one column group in thread order
+            constexpr int GU = NW / 8;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sRed[tid * 8 + k] = cs[k];
+            named_sync(1, kProducers);
+            for (int c = tid; c < N; c += kProducers) {
+                float s = 0.f;
+                for (int i = c / 8; i < kProducers; i += GU) s += sRed[i * 8 + (c & 7)];
+                part[(int64_t)N * K + c] = s;
+            }
+        }
+    } else if (warp == kProducerWarps + kEpilogueWarps) {
+        if (lane == 0) {
+            const uint32_t gb = smem_u32(sm + P.g), hb = smem_u32(sm + P.h);
+            const uint64_t gk = kmajor_desc(gb, 128, Sg, 0), wk = kmajor_desc(smem_u32(sm + P.w), KW, Sg, 0);
+            const uint64_t gm = sdesc(gb, 128u * Sg, 8 * Sg, swz_code(Sg)), hm = sdesc(hb, 128u * Sh, 8 * Sh, swz_code(Sh));
+            constexpr uint32_t id1 = idesc_bf16(128, KW), id2 = idesc_bf16(128, KW, 1, 1);
+            bool ok = true;
+            int j = 0;
+            for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++j) {
+                const int b = j & 1;
+                const uint32_t go = (uint32_t)b * 3 * P.gterm, par = (uint32_t)((j >> 1) - 1) & 1u;
+                if (j >= 2) ok = mbar_wait(acc_empty + b, par);
+                ok = ok && mbar_wait(full_g + b, (uint32_t)(j >> 1) & 1u);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t d = tmem + (uint32_t)(b * 2 * KW);
+#pragma unroll
+                for (int p = 0; p < 6; ++p) {
+                    const uint64_t a = desc_step(gk, go + kTermA[p] * P.gterm), w = desc_step(wk, kTermB[p] * P.wterm);
+#pragma unroll
+                    for (int k0 = 0; k0 < NW; k0 += 16)
+                        mma_bf16(p < 5 ? d + KW : d, desc_step(a, k0 * 2), desc_step(w, k0 * 2), id1,
+                                 ((p > 0 && p < 5) || k0 > 0) ? 1u : 0u);
+                }
+                mma_commit(acc_full + b);
+                if (j >= 2) ok = mbar_wait(w_empty + b, par);
+                ok = ok && mbar_wait(full_h, (uint32_t)j & 1u);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t dw = tmem + WCOL + (uint32_t)(b * KW);
+#pragma unroll
+                for (int p = 0; p < 6; ++p) {
+                    const uint64_t a = desc_step(gm, go + kTermA[p] * P.gterm), h = desc_step(hm, kTermB[p] * P.hterm);
+#pragma unroll
+                    for (int k0 = 0; k0 < 128; k0 += 16)
+                        mma_bf16(dw, desc_step(a, (uint32_t)(k0 * Sg)), desc_step(h, (uint32_t)(k0 * Sh)), id2,
+                                 (p > 0 || k0 > 0) ? 1u : 0u);
+                }
+                mma_commit(empty_g + b);
+                mma_commit(empty_h);
+                mma_commit(w_full + b);
+            }
+            // the last releases have arrived before the block may end
+            if (ok && j > 0) {
+                mbar_wait(empty_h, (uint32_t)(j - 1) & 1u);
+                mbar_wait(empty_g + ((j - 1) & 1), (uint32_t)((j - 1) >> 1) & 1u);
+            }
+        }
+        __syncwarp();
+    } else {
+        const int ew = warp - kProducerWarps, eg = ew >> 2, q = ew & 3;
+        float* stg = reinterpret_cast<float*>(sm + P.stg + ew * kStageBytes);
+        const uint32_t lane_base = (uint32_t)(32 * q) << 16;
+        const int rs = lane >> 2, c4 = (lane & 3) * 4;
+        const int c0w = eg * CW;               // this thread's dW columns (row 32 q + lane)
+        float acc[CW];
+#pragma unroll
+        for (int i = 0; i < CW; ++i) acc[i] = 0.f;
+        bool ok = true;
+        int j = 0;
+        for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++j) {
+            const int b = j & 1;
+            if (b == eg) {   // this group's tile: dz' = acc ELU'(h)
+                const int64_t rb = (int64_t)t * 128 + 32 * q;
+                const int nv = (int)std::min<int64_t>(32, std::max<int64_t>(0, A.rows - rb));
+                int64_t row[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) row[i] = nv > 0 ? rb + std::min(8 * i + rs, nv - 1) : 0;
+                auto load_h = [&](int c0, float4* x) {
+                    const int nc = K - (c0 + c4), col = VEC ? std::min(c0 + c4, K - 4) : c0 + c4;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) x[i] = load4<VEC>(A.H + row[i] * K + col, VEC ? 4 : nc);
+                };
+                float4 x[4];
+                load_h(0, x);
+                ok = warp_wait(acc_full + b, (uint32_t)(j >> 1) & 1u, lane);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t tacc = tmem + lane_base + (uint32_t)(b * 2 * KW);
+#pragma unroll
+                for (int c0 = 0; c0 < KW; c0 += 16) {
+                    float v[16];
+                    load_sum16(tacc + c0, KW, v);
+#pragma unroll
+                    for (int i = 0; i < 16; i += 4)
+                        *reinterpret_cast<float4*>(stg + lane * kStageLd + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                    __syncwarp();
+                    float4 u[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 z = *reinterpret_cast<const float4*>(stg + (8 * i + rs) * kStageLd + c4);
+                        u[i] = make_float4(z.x * elu1_deriv_from_out(x[i].x), z.y * elu1_deriv_from_out(x[i].y),
+                                           z.z * elu1_deriv_from_out(x[i].z), z.w * elu1_deriv_from_out(x[i].w));
+                    }
+                    if (c0 + 16 < KW) load_h(c0 + 16, x);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (8 * i + rs < nv) store4<VEC>(A.out + row[i] * K + c0 + c4, K - (c0 + c4), u[i]);
+                    __syncwarp();
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(acc_empty + b);
+            }
+            ok = warp_wait(w_full + b, (uint32_t)(j >> 1) & 1u, lane);
+            if (!ok) break;
+            tc_fence_after();
+            if (c0w < KW) {
+#pragma unroll
+                for (int i = 0; i < CW; i += 16) {
+                    float v[16];
+                    tmem_ld16(tmem + lane_base + WCOL + (uint32_t)(b * KW + c0w + i), v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) acc[i + k] += v[k];
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(w_empty + b);
+        }
+        const int r = 32 * q + lane;
+        if (c0w < KW && r < N) {
+#pragma unroll
+            for (int i = 0; i < CW; ++i)
+                if (c0w + i < K) part[(int64_t)r * K + c0w + i] = acc[i];
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0) tmem_dealloc(tmem, NCOLS);
+}
+
 // ------------------------------------------------------------------ k_reduce3
 
 struct RedArgs {
@@ -1032,6 +1347,49 @@ int wgrad(int64_t rows, const float* G, int64_t ldg, int N, const float* X, int6
     else launch(k_wgrad3<128>);
     if (rc) return rc;
     GNN_LAUNCH_CHECK("k_wgrad3");
+    return GNN_OK;
+}
+
+bool chain_fits(int N, int K) { return N <= 64 && K <= 64; }
+
+int chain(int64_t rows, const float* G, int N, const float* H, int K, const float* W, float* out, bool db, float* part,
+          cudaStream_t s, int* ctas) {
+    *ctas = 0;
+    if (rows == 0) return GNN_OK;
+    GNN_REQUIRE(chain_fits(N, K), GNN_EUNSUPPORTED, "lin3: chain %d x %d does not fit", N, K);
+    CArgs a{};
+    a.rows = rows;
+    const int64_t nt = (rows + 127) / 128;
+    GNN_REQUIRE(nt <= 0x7fffffff - 2 * kMaxCtas, GNN_ESHAPE, "lin3: too many rows");
+    a.n_tiles = (int)nt;
+    a.G = G; a.N = N;
+    a.H = H; a.K = K;
+    a.W = W; a.out = out; a.db = db ? 1 : 0; a.part = part;
+    const bool vec = N % 4 == 0 && K % 4 == 0 && aligned16(G) && aligned16(H) && aligned16(out);
+    const int grid = (int)std::min<int64_t>(nt, std::min(kMaxCtas, fused::host::num_sms()));
+    *ctas = grid;
+    int rc = GNN_OK;
+    auto launch = [&](auto nw, auto kw) {
+        constexpr int NW = decltype(nw)::value, KW = decltype(kw)::value;
+        constexpr uint32_t smem = chain_smem<NW, KW>().total;
+        static_assert(smem <= kSmemMax, "one block per SM");
+        auto kern = vec ? k_chain3<NW, KW, true> : k_chain3<NW, KW, false>;
+        if ((rc = set_smem(kern, smem))) return;
+        ProfScope _ps(s, "k_chain3");
+        kern<<<grid, kThreads, smem, s>>>(a);
+    };
+    auto with_k = [&](auto nw) {
+        const int kw = pow2_width(K);
+        if (kw == 16) launch(nw, Int<16>());
+        else if (kw == 32) launch(nw, Int<32>());
+        else launch(nw, Int<64>());
+    };
+    const int nw = pow2_width(N);
+    if (nw == 16) with_k(Int<16>());
+    else if (nw == 32) with_k(Int<32>());
+    else with_k(Int<64>());
+    if (rc) return rc;
+    GNN_LAUNCH_CHECK("k_chain3");
     return GNN_OK;
 }
 

@@ -64,6 +64,12 @@ int wgrad(int64_t rows, const float* G, int64_t ldg, int N, const float* X, int6
           cudaStream_t s, int* ctas);
 inline int64_t wgrad_floats(int N, int K) { return (int64_t)kMaxCtas * (N * K + N); }
 
+// out [rows x K] = (G W) ELU'(H) and the partials of wgrad(G, H) in one pass
+// (G [rows x N], H = ELU outputs [rows x K], W [N x K], all dense).
+bool chain_fits(int N, int K);
+int chain(int64_t rows, const float* G, int N, const float* H, int K, const float* W, float* out, bool db, float* part,
+          cudaStream_t s, int* ctas);
+
 // dst[n * ldd + k] += sum over z of part[z * stride + n * K + k], z ascending per lane.
 struct Sum {
     const float* part;

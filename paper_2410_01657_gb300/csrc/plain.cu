@@ -819,6 +819,18 @@ struct GradSums {
         part += lin3::wgrad_floats(N, K);
         return GNN_OK;
     }
+    // the same with X = ELU outputs, and out = (G W) ELU'(X), in one pass
+    int chain(int64_t rows, const float* G, int N, const float* X, int K, const float* W, float* out, float* dW,
+              float* db, cudaStream_t st) {
+        int nz = 0;
+        int rc = lin3::chain(rows, G, N, X, K, W, out, true, part, st, &nz);
+        if (rc) return rc;
+        const int64_t stride = (int64_t)N * K + N;
+        s[n++] = {part, stride, nz, N, K, dW, K};
+        s[n++] = {part + (int64_t)N * K, stride, nz, 1, N, db, N};
+        part += lin3::wgrad_floats(N, K);
+        return GNN_OK;
+    }
 };
 static int64_t tc_grad_floats(const gnn_mlp& P, int in, int sources) {
     int64_t f = (int64_t)lin3::kMaxCtas * 2 * P.dims[P.n_lin] + sources * lin3::wgrad_floats(P.dims[1], in);
@@ -852,6 +864,12 @@ static int tc_chain_bwd(const gnn_mlp& P, const gnn_mlp& dP, int64_t rows, float
     float* next = g == g0 ? g1 : g0;
     for (int k = n - 1; k >= 1; --k) {
         const int N = P.dims[k + 1], K = P.dims[k];
+        if (lin3::chain_fits(N, K)) {
+            if ((rc = gs.chain(rows, g, N, hbuf[k], K, P.W[k], next, dP.W[k], dP.b[k], s))) return rc;
+            g = next;
+            next = g == g0 ? g1 : g0;
+            continue;
+        }
         if ((rc = gs.weight(rows, g, N, hbuf[k], K, K, dP.W[k], K, dP.b[k], s))) return rc;
         lin3::Args a = dgrad_args(rows, g, N, P.W[k], K, K, next, K);
         a.add = hbuf[k]; a.ldadd = K;
