@@ -1308,20 +1308,25 @@ __global__ void __launch_bounds__(Cfg<H>::NT) k_node_fwd(const __grid_constant__
             // whole by one warp (lane l: columns 4l .. 4l+3; warp w: rows 8w .. 8w+7); the x
             // rows wait in registers until the a* half has been multiplied
             static_assert(C::NT == 512 && H == 128, "row-per-warp fill: 16 warps x 8 rows, 32 lanes x 4 columns");
-            float4 xr[8];
+            uint2 ar[8], xr[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const int rr = 8 * warp + i;
-                const int64_t rg = t * 128 + rr;
-                float4 av = make_float4(0.f, 0.f, 0.f, 0.f);
-                xr[i] = av;
+                const int64_t rg = t * 128 + 8 * warp + i;
+                float4 av = make_float4(0.f, 0.f, 0.f, 0.f), xw = av;
                 if (rg < A.n_rows) {
                     av = __ldg(reinterpret_cast<const float4*>(A.a_star + rg * H) + lane);
-                    xr[i] = __ldg(reinterpret_cast<const float4*>(A.x + rg * H) + lane);
+                    xw = __ldg(reinterpret_cast<const float4*>(A.x + rg * H) + lane);
                 }
-                *reinterpret_cast<uint2*>(sA0 + tile_off(rr, 4 * lane, 128, C::S)) =
-                    make_uint2(pack_bf16x2(av.x, av.y), pack_bf16x2(av.z, av.w));
+                ar[i] = make_uint2(pack_bf16x2(av.x, av.y), pack_bf16x2(av.z, av.w));
+                xr[i] = make_uint2(pack_bf16x2(xw.x, xw.y), pack_bf16x2(xw.z, xw.w));
             }
+            if constexpr (SAVE) {   // the chain's tile is this buffer: the previous tile's dz store has to have read it
+                if (tid == 0) bulk_wait_read_all();
+                __syncthreads();
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                *reinterpret_cast<uint2*>(sA0 + tile_off(8 * warp + i, 4 * lane, 128, C::S)) = ar[i];
             fence_proxy_async();
             tc_fence_before();
             __syncthreads();
@@ -1343,8 +1348,7 @@ __global__ void __launch_bounds__(Cfg<H>::NT) k_node_fwd(const __grid_constant__
             if (!ok) break;
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-                *reinterpret_cast<uint2*>(sA0 + tile_off(8 * warp + i, 4 * lane, 128, C::S)) =
-                    make_uint2(pack_bf16x2(xr[i].x, xr[i].y), pack_bf16x2(xr[i].z, xr[i].w));
+                *reinterpret_cast<uint2*>(sA0 + tile_off(8 * warp + i, 4 * lane, 128, C::S)) = xr[i];
             fence_proxy_async();
             tc_fence_before();
             __syncthreads();
