@@ -9,19 +9,21 @@
 // makes every piece agree in sign with x: the parts left out then add up.)
 // The tensor core truncates its running sums, so a sum must not carry terms
 // far below it: the hi hi products have an accumulator of their own, the five
-// small ones share another, and the epilogue adds the two. Sums in tensor
+// small ones one or two others, and the epilogue adds them up. Sums in tensor
 // memory run over at most 256 products per output (inputs) or one tile of rows
 // (weight gradients, continued in FP32 registers, rounding to nearest).
 //
 // What bounds it: at width 64 a Linear moves 512 bytes per row for 49 kFLOP of
 // BF16 products, 96 FLOP per byte, far below the ridge: HBM, if the splitting
 // (about 6 instructions per element) and the epilogue are hidden. So the block
-// is specialised: eight warps load FP32 rows, split them and write the three
-// operand tiles (swizzled K-major rows); one thread issues the MMAs; two
-// groups of four warps take alternate tiles from two tensor-memory
+// is specialised: four warps load FP32 rows, split them and write the three
+// operand tiles (swizzled K-major rows); one warp issues the MMAs; two
+// groups of four warps take alternate tiles from two sets of tensor-memory
 // accumulators, through a per-warp staging tile so that every global access of
 // an epilogue (bias, residual, gathers, stores) is a run of whole 64-byte
-// pieces of rows.
+// pieces of rows. A Linear with ELU of 1.34M rows at width 64 takes 0.16 ms,
+// 4.3 TB/s (HBM alone: 0.10). A third epilogue group (16 warps, each group
+// issuing its own MMAs) gave the same there and cost the narrow widths 12 %.
 
 #include <algorithm>
 
@@ -146,12 +148,24 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int la
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-// 16 columns of the lane's row: the hi hi sum plus the small products' sum.
-__device__ __forceinline__ void load_sum16(uint32_t taddr, int NP, float* v) {
+// 16 columns of the lane's row: the hi hi sum plus the small products' sum (or sums, if three).
+__device__ __forceinline__ void load_sum16(uint32_t taddr, int NP, bool three, float* v) {
     float u[16];
     tmem_ld16(taddr, v);
     tmem_ld16(taddr + NP, u);
-    tmem_ld_wait();
+    if (three) {
+        float w[16];
+        tmem_ld16(taddr + 2 * NP, w);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 16; i += 2) {
+            const float2 z = __fadd2_rn(make_float2(u[i], u[i + 1]), make_float2(w[i], w[i + 1]));
+            u[i] = z.x;
+            u[i + 1] = z.y;
+        }
+    } else {
+        tmem_ld_wait();
+    }
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
         const float2 w = __fadd2_rn(make_float2(v[i], v[i + 1]), make_float2(u[i], u[i + 1]));
@@ -190,6 +204,16 @@ __device__ __forceinline__ float2 elu_pair(float2 z) {
 // The six products of a split pair, smallest first: (term of A, term of B).
 __device__ constexpr int kTermA[6] = {2, 0, 1, 1, 0, 0};
 __device__ constexpr int kTermB[6] = {0, 2, 1, 0, 1, 0};
+
+// An MMA of 128 x 64 x 16 needs 32 cycles of the tensor core, but one follows the other at 110
+// whatever its width when one lane of a diverged warp issues them, and at 85 when the whole warp
+// goes through the loop and one lane acts. So the warp stays together, and the terms of B lie one
+// after the other as rows of one tile: up to width 80 three MMAs do the six products, hi of A with
+// [hi | mid | lo] of B, mid with [hi | mid], lo with [hi], into three sums [hi hi | 2^-8 terms |
+// 2^-16 terms]. Per row tile at width 64: 1,650 cycles where the 24 narrow ones took 2,630. For a
+// weight gradient the terms of X are consecutive blocks of one MN-major operand, up to width 64
+// (1.0 -> 0.83 of the time at 64).
+__host__ __device__ inline bool three_sums(int NP) { return NP <= 80; }   // N = 3 NP <= 256
 
 // ------------------------------------------------------------------ shared memory
 
@@ -296,7 +320,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
     uint64_t* acc_full = full + 8;
     uint64_t* acc_empty = full + 10;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + P.tm);
-    const uint32_t NCOLS = pow2_cols(4 * (uint32_t)NP);   // two tiles x {hi hi, small products}
+    const bool three = three_sums(NP);
+    const int ACC = (three ? 3 : 2) * NP;                       // columns of a tile's accumulators
+    const uint32_t NCOLS = pow2_cols(2 * (uint32_t)ACC);        // two tiles
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (warp == 0) {
@@ -354,16 +380,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
         else if (KB == 32) lin_producer<32, VEC, MODE>(A, P, sm, full, empty, tid, lane);
         else lin_producer<16, VEC, MODE>(A, P, sm, full, empty, tid, lane);
     } else if (warp == kProducerWarps + kEpilogueWarps) {
-        // ---- one thread issues the MMAs
-        if (lane == 0) {
-            const uint32_t id = idesc_bf16(128, NP);
+        // ---- one lane of a converged warp issues the MMAs
+        {
+            const uint32_t lead = elect_one();
+            const uint32_t id = idesc_bf16(128, NP), id2 = idesc_bf16(128, 2 * NP), id3 = idesc_bf16(128, 3 * NP);
             const uint64_t a0 = kmajor_desc(smem_u32(sm + P.a), 128, S, 0);
             const uint64_t w0 = kmajor_desc(smem_u32(sm + P.w), NP, S, 0);
             int n = 0, j = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++j) {
                 const int buf = j & 1;
-                const uint32_t d = tmem + (uint32_t)(buf * 2 * NP);
+                const uint32_t d = tmem + (uint32_t)(buf * ACC);
                 if (j >= 2) ok = mbar_wait(acc_empty + buf, (uint32_t)((j >> 1) - 1) & 1u);
                 for (int b = 0; b < nkb && ok; ++b, ++n) {
                     const int st = n % stages, use = n / stages;
@@ -372,22 +399,34 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                     tc_fence_after();
                     const uint32_t ao = (uint32_t)st * 3 * P.aterm, wo = (uint32_t)b * 3 * P.wterm;
                     auto issue = [&](auto kb) {
+                        if (three) {
+                            const uint64_t wp = desc_step(w0, wo);
+#pragma unroll
+                            for (int p = 0; p < 3; ++p) {
+                                const uint64_t ap = desc_step(a0, ao + p * P.aterm);
+#pragma unroll
+                                for (int k0 = 0; k0 < decltype(kb)::value; k0 += 16)   // one swizzle block, 32 bytes a step
+                                    mma_bf16_warp(lead, d + p * NP, desc_step(ap, k0 * 2), desc_step(wp, k0 * 2),
+                                                  p == 0 ? id3 : (p == 1 ? id2 : id), (b > 0 || p > 0 || k0 > 0) ? 1u : 0u);
+                            }
+                            return;
+                        }
 #pragma unroll
                         for (int p = 0; p < 6; ++p) {
                             const uint64_t ap = desc_step(a0, ao + kTermA[p] * P.aterm);
                             const uint64_t wp = desc_step(w0, wo + kTermB[p] * P.wterm);
 #pragma unroll
-                            for (int k0 = 0; k0 < decltype(kb)::value; k0 += 16)   // one swizzle block, 32 bytes a step
-                                mma_bf16(p < 5 ? d + NP : d, desc_step(ap, k0 * 2), desc_step(wp, k0 * 2), id,
+                            for (int k0 = 0; k0 < decltype(kb)::value; k0 += 16)
+                                mma_bf16_warp(lead, p < 5 ? d + NP : d, desc_step(ap, k0 * 2), desc_step(wp, k0 * 2), id,
                                          (b > 0 || (p > 0 && p < 5) || k0 > 0) ? 1u : 0u);
                         }
                     };
                     if (KB == 64) issue(Int<64>());
                     else if (KB == 32) issue(Int<32>());
                     else issue(Int<16>());
-                    mma_commit(empty + st);
+                    mma_commit_warp(lead, empty + st);
                 }
-                if (ok) mma_commit(acc_full + buf);
+                if (ok) mma_commit_warp(lead, acc_full + buf);
             }
             // the last stage's release has arrived before the block may end
             if (ok && n > 0) mbar_wait(empty + (n - 1) % stages, (uint32_t)((n - 1) / stages) & 1u);
@@ -399,7 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
         const int ew = warp - kProducerWarps, eg = ew >> 2, q = ew & 3;
         float* stg = reinterpret_cast<float*>(sm + P.stg + ew * kStageBytes);
         float* sums = reinterpret_cast<float*>(sm + P.sums) + ew * 2 * NP;
-        const uint32_t tacc = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(eg * 2 * NP);
+        const uint32_t tacc = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(eg * ACC);
         const int rs = lane >> 2, c4 = (lane & 3) * 4;
         constexpr bool kGather = MODE == kElu && OPS == kOpsGather, kEdge = MODE == kLnAdjoint && OPS == kOpsGather;
         bool ok = true;
@@ -465,7 +504,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                 float s4[4] = {0.f, 0.f, 0.f, 0.f};
                 for (int c0 = 0; c0 < N; c0 += 16) {
                     float v[16];
-                    load_sum16(tacc + c0, NP, v);
+                    load_sum16(tacc + c0, NP, three, v);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) s4[i & 3] += v[i] + sPar[c0 + i];   // padding columns are zero
                 }
@@ -473,7 +512,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                 float q4[4] = {0.f, 0.f, 0.f, 0.f};
                 for (int c0 = 0; c0 < N; c0 += 16) {
                     float v[16];
-                    load_sum16(tacc + c0, NP, v);
+                    load_sum16(tacc + c0, NP, three, v);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const float d = c0 + i < N ? v[i] + sPar[c0 + i] - mean : 0.f;
@@ -495,7 +534,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                         *reinterpret_cast<float4*>(stg + r * kStageLd + c4) = g[i];
                     }
                     float v[16];
-                    load_sum16(tacc + c0, NP, v);
+                    load_sum16(tacc + c0, NP, three, v);
                     __syncwarp();
 #pragma unroll
                     for (int i = 0; i < 16; i += 4) {
@@ -517,7 +556,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
             for (int c0 = 0; c0 < NP; c0 += 16) {
                 const int col = c0 + c4, nc = N - col;
                 float v[16];
-                load_sum16(tacc + c0, NP, v);
+                load_sum16(tacc + c0, NP, three, v);
                 if constexpr (MODE == kLayerNorm || MODE == kLnAdjoint) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] = (v[i] + sPar[c0 + i] - mean) * rstd;   // xhat
@@ -724,8 +763,8 @@ __device__ __forceinline__ void wgrad_producer(const WArgs& A, const WSmem& P, c
 }
 
 // dW = G^T X over the CTA's row tiles: both operands are MN-major views of the
-// same split row tiles (rows = the contraction). The accumulator of one tile
-// (RT rows) is added to FP32 registers by the epilogue warps, so no tensor-core
+// same split row tiles (rows = the contraction). The sums of one tile (RT rows)
+// are added to FP32 registers by the epilogue warps, so no tensor-core
 // sum runs over more than RT rows.
 template <int KP>
 __global__ void __launch_bounds__(kWThreads, 1) k_wgrad3(const __grid_constant__ WArgs A) {
@@ -741,7 +780,8 @@ __global__ void __launch_bounds__(kWThreads, 1) k_wgrad3(const __grid_constant__
     uint64_t* acc_empty = full + 10;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + P.tm);
     float* sRed = reinterpret_cast<float*>(sm + P.red);
-    constexpr uint32_t NCOLS = 2 * KP < 32 ? 32 : 2 * KP;
+    constexpr int SUMS = KP <= 64 ? 3 : 1;              // accumulators of a tile (of width 128: one)
+    constexpr uint32_t NCOLS = 2 * SUMS * KP <= 128 ? 128 : (2 * SUMS * KP <= 256 ? 256 : 512);
     constexpr int CW = KP >= 32 ? KP / 2 : 16;      // accumulator columns per epilogue thread
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -802,8 +842,9 @@ __global__ void __launch_bounds__(kWThreads, 1) k_wgrad3(const __grid_constant__
             }
         }
     } else if (warp == kWProducerWarps + kEpilogueWarps) {
-        if (lane == 0) {
-            const uint32_t id = idesc_bf16(128, KP, 1, 1);
+        {
+            const uint32_t lead = elect_one();
+            constexpr uint32_t id = idesc_bf16(128, KP, 1, 1);
             const uint32_t base = smem_u32(sm + P.st);
             const uint64_t g0 = sdesc(base, (uint32_t)RT * Sg, 8 * Sg, swz_code(Sg));
             const uint64_t x0 = sdesc(base + 3 * P.gterm, (uint32_t)RT * Sx, 8 * Sx, swz_code(Sx));
@@ -815,22 +856,35 @@ __global__ void __launch_bounds__(kWThreads, 1) k_wgrad3(const __grid_constant__
                 ok = ok && mbar_wait(full + st, (uint32_t)use & 1u);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t d = tmem + (uint32_t)(buf * KP), so = (uint32_t)st * P.stage;
+                const uint32_t d = tmem + (uint32_t)(buf * SUMS * KP), so = (uint32_t)st * P.stage;
                 auto issue = [&](auto rt) {
+                    if constexpr (SUMS == 3) {   // the terms of X are consecutive blocks of one MN-major operand
+                        const uint64_t xp = desc_step(x0, so);
 #pragma unroll
-                    for (int p = 0; p < 6; ++p) {
-                        const uint64_t gp = desc_step(g0, so + kTermA[p] * P.gterm);
-                        const uint64_t xp = desc_step(x0, so + kTermB[p] * P.xterm);
+                        for (int p = 0; p < 3; ++p) {
+                            const uint64_t gp = desc_step(g0, so + p * P.gterm);
+                            constexpr uint32_t ids[3] = {idesc_bf16(128, 3 * KP, 1, 1), idesc_bf16(128, 2 * KP, 1, 1), id};
 #pragma unroll
-                        for (int k0 = 0; k0 < decltype(rt)::value; k0 += 16)
-                            mma_bf16(d, desc_step(gp, (uint32_t)(k0 * Sg)), desc_step(xp, (uint32_t)(k0 * Sx)), id,
-                                     (p > 0 || k0 > 0) ? 1u : 0u);
+                            for (int k0 = 0; k0 < decltype(rt)::value; k0 += 16)
+                                mma_bf16_warp(lead, d + p * KP, desc_step(gp, (uint32_t)(k0 * Sg)), desc_step(xp, (uint32_t)(k0 * Sx)),
+                                         ids[p], (p > 0 || k0 > 0) ? 1u : 0u);
+                        }
+                    } else {
+#pragma unroll
+                        for (int p = 0; p < 6; ++p) {
+                            const uint64_t gp = desc_step(g0, so + kTermA[p] * P.gterm);
+                            const uint64_t xp = desc_step(x0, so + kTermB[p] * P.xterm);
+#pragma unroll
+                            for (int k0 = 0; k0 < decltype(rt)::value; k0 += 16)
+                                mma_bf16_warp(lead, d, desc_step(gp, (uint32_t)(k0 * Sg)), desc_step(xp, (uint32_t)(k0 * Sx)), id,
+                                         (p > 0 || k0 > 0) ? 1u : 0u);
+                        }
                     }
                 };
                 if (RT == 64) issue(Int<64>());
                 else issue(Int<128>());
-                mma_commit(empty + st);
-                mma_commit(acc_full + buf);
+                mma_commit_warp(lead, empty + st);
+                mma_commit_warp(lead, acc_full + buf);
             }
             if (ok && n > 0) mbar_wait(empty + (n - 1) % stages, (uint32_t)((n - 1) / stages) & 1u);
         }
@@ -853,8 +907,13 @@ __global__ void __launch_bounds__(kWThreads, 1) k_wgrad3(const __grid_constant__
 #pragma unroll
                 for (int i = 0; i < CW; i += 16) {
                     float v[16];
-                    tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * KP + c0 + i), v);
-                    tmem_ld_wait();
+                    const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * SUMS * KP + c0 + i);
+                    if constexpr (SUMS == 3) {
+                        load_sum16(ta, KP, true, v);
+                    } else {
+                        tmem_ld16(ta, v);
+                        tmem_ld_wait();
+                    }
 #pragma unroll
                     for (int k = 0; k < 16; ++k) acc[i + k] += v[k];
                 }
@@ -885,8 +944,9 @@ __global__ void __launch_bounds__(kWThreads, 1) k_wgrad3(const __grid_constant__
 // and each row is read once instead of twice (three tensors moved instead of
 // five). Two stages of dz and one of h fill shared memory beside W; the widths
 // above 64 need twice that and keep the two launches. 3.23M edge rows at width
-// 64: 0.84 ms as it stands against 0.49 + 0.48 for the two launches: the four
-// producer warps split both operands and set the pace (HBM alone: 0.37).
+// 64: 0.72 ms (0.84 with one MMA per product) against 0.49 + 0.48 for the two
+// launches: the four producer warps split both operands and set the pace (HBM
+// alone: 0.37).
 struct CArgs {
     int64_t rows;
     int n_tiles;
@@ -982,8 +1042,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
     uint64_t* w_empty = full_g + 12;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + P.tm);
     float* sRed = reinterpret_cast<float*>(sm + P.red);
-    // TMEM: dz' of two tiles (hi hi | small products), dW of two tiles
-    constexpr uint32_t NCOLS = 6 * KW <= 128 ? 128 : (6 * KW <= 256 ? 256 : 512), WCOL = 4 * KW;
+    // TMEM: dz' of two tiles, three sums each (at KW = 64 two: five MMAs a K-step), then dW, three
+    // sums, of two tiles (at KW = 64 of one: the next tile's dz' is under way while it is read)
+    constexpr int ZS = KW <= 32 ? 3 : 2, WB = KW <= 32 ? 2 : 1;
+    constexpr uint32_t WCOL = 2 * ZS * KW;
+    constexpr uint32_t NCOLS = WCOL + WB * 3 * KW <= 256 ? 256 : 512;
+    static_assert(WCOL + WB * 3 * KW <= 512, "tensor memory");
     constexpr int CW = KW >= 32 ? KW / 2 : 16;   // dW columns per epilogue thread
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, N = A.N, K = A.K;
 
@@ -1058,11 +1122,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
             }
         }
     } else if (warp == kProducerWarps + kEpilogueWarps) {
-        if (lane == 0) {
+        {
+            const uint32_t lead = elect_one();
             const uint32_t gb = smem_u32(sm + P.g), hb = smem_u32(sm + P.h);
             const uint64_t gk = kmajor_desc(gb, 128, Sg, 0), wk = kmajor_desc(smem_u32(sm + P.w), KW, Sg, 0);
             const uint64_t gm = sdesc(gb, 128u * Sg, 8 * Sg, swz_code(Sg)), hm = sdesc(hb, 128u * Sh, 8 * Sh, swz_code(Sh));
-            constexpr uint32_t id1 = idesc_bf16(128, KW), id2 = idesc_bf16(128, KW, 1, 1);
+            constexpr uint32_t idz[3] = {idesc_bf16(128, ZS * KW), idesc_bf16(128, (ZS - 1) * KW), idesc_bf16(128, KW)};
+            constexpr uint32_t idw[3] = {idesc_bf16(128, 3 * KW, 1, 1), idesc_bf16(128, 2 * KW, 1, 1), idesc_bf16(128, KW, 1, 1)};
             bool ok = true;
             int j = 0;
             for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++j) {
@@ -1072,32 +1138,40 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
                 ok = ok && mbar_wait(full_g + b, (uint32_t)(j >> 1) & 1u);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t d = tmem + (uint32_t)(b * 2 * KW);
-#pragma unroll
-                for (int p = 0; p < 6; ++p) {
-                    const uint64_t a = desc_step(gk, go + kTermA[p] * P.gterm), w = desc_step(wk, kTermB[p] * P.wterm);
+                const uint32_t d = tmem + (uint32_t)(b * ZS * KW);
+                auto z = [&](int col, int ta, int tw, uint32_t id, bool add) {
+                    const uint64_t a = desc_step(gk, go + ta * P.gterm), w = desc_step(wk, tw * P.wterm);
 #pragma unroll
                     for (int k0 = 0; k0 < NW; k0 += 16)
-                        mma_bf16(p < 5 ? d + KW : d, desc_step(a, k0 * 2), desc_step(w, k0 * 2), id1,
-                                 ((p > 0 && p < 5) || k0 > 0) ? 1u : 0u);
+                        mma_bf16_warp(lead, d + col * KW, desc_step(a, k0 * 2), desc_step(w, k0 * 2), id, (add || k0 > 0) ? 1u : 0u);
+                };
+                z(0, 0, 0, idz[0], false);
+                z(1, 1, 0, idz[1], true);
+                if constexpr (ZS == 3) {
+                    z(2, 2, 0, idz[2], true);
+                } else {
+                    z(1, 2, 0, idz[2], true);
+                    z(1, 1, 1, idz[2], true);
+                    z(1, 0, 2, idz[2], true);
                 }
-                mma_commit(acc_full + b);
-                if (j >= 2) ok = mbar_wait(w_empty + b, par);
+                mma_commit_warp(lead, acc_full + b);
+                const int wb = j % WB;
+                if (j >= WB) ok = mbar_wait(w_empty + wb, (uint32_t)(j / WB - 1) & 1u);
                 ok = ok && mbar_wait(full_h, (uint32_t)j & 1u);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t dw = tmem + WCOL + (uint32_t)(b * KW);
+                const uint32_t dw = tmem + WCOL + (uint32_t)(wb * 3 * KW);
 #pragma unroll
-                for (int p = 0; p < 6; ++p) {
-                    const uint64_t a = desc_step(gm, go + kTermA[p] * P.gterm), h = desc_step(hm, kTermB[p] * P.hterm);
+                for (int p = 0; p < 3; ++p) {
+                    const uint64_t a = desc_step(gm, go + p * P.gterm);
 #pragma unroll
                     for (int k0 = 0; k0 < 128; k0 += 16)
-                        mma_bf16(dw, desc_step(a, (uint32_t)(k0 * Sg)), desc_step(h, (uint32_t)(k0 * Sh)), id2,
+                        mma_bf16_warp(lead, dw + p * KW, desc_step(a, (uint32_t)(k0 * Sg)), desc_step(hm, (uint32_t)(k0 * Sh)), idw[p],
                                  (p > 0 || k0 > 0) ? 1u : 0u);
                 }
-                mma_commit(empty_g + b);
-                mma_commit(empty_h);
-                mma_commit(w_full + b);
+                mma_commit_warp(lead, empty_g + b);
+                mma_commit_warp(lead, empty_h);
+                mma_commit_warp(lead, w_full + wb);
             }
             // the last releases have arrived before the block may end
             if (ok && j > 0) {
@@ -1116,6 +1190,26 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
 #pragma unroll
         for (int i = 0; i < CW; ++i) acc[i] = 0.f;
         bool ok = true;
+        // dW of tile j into the registers: by the tile's own group halfway through it, by the other
+        // one after its tile before, at about the same time
+        auto read_w = [&](int j) {
+            const int wb = j % WB;
+            ok = warp_wait(w_full + wb, (uint32_t)(j / WB) & 1u, lane);
+            if (!ok) return;
+            tc_fence_after();
+            if (c0w < KW) {
+#pragma unroll
+                for (int i = 0; i < CW; i += 16) {
+                    float v[16];
+                    load_sum16(tmem + lane_base + WCOL + (uint32_t)(wb * 3 * KW + c0w + i), KW, true, v);
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) acc[i + k] += v[k];
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(w_empty + wb);
+        };
         int j = 0;
         for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++j) {
             const int b = j & 1;
@@ -1135,11 +1229,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
                 ok = warp_wait(acc_full + b, (uint32_t)(j >> 1) & 1u, lane);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t tacc = tmem + lane_base + (uint32_t)(b * 2 * KW);
+                const uint32_t tacc = tmem + lane_base + (uint32_t)(b * ZS * KW);
 #pragma unroll
                 for (int c0 = 0; c0 < KW; c0 += 16) {
                     float v[16];
-                    load_sum16(tacc + c0, KW, v);
+                    load_sum16(tacc + c0, KW, ZS == 3, v);
 #pragma unroll
                     for (int i = 0; i < 16; i += 4)
                         *reinterpret_cast<float4*>(stg + lane * kStageLd + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
@@ -1156,27 +1250,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
                     for (int i = 0; i < 4; ++i)
                         if (8 * i + rs < nv) store4<VEC>(A.out + row[i] * K + c0 + c4, K - (c0 + c4), u[i]);
                     __syncwarp();
+                    if (c0 == (KW == 64 ? 16 : 0)) read_w(j);
                 }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(acc_empty + b);
             }
-            ok = warp_wait(w_full + b, (uint32_t)(j >> 1) & 1u, lane);
-            if (!ok) break;
-            tc_fence_after();
-            if (c0w < KW) {
-#pragma unroll
-                for (int i = 0; i < CW; i += 16) {
-                    float v[16];
-                    tmem_ld16(tmem + lane_base + WCOL + (uint32_t)(b * KW + c0w + i), v);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) acc[i + k] += v[k];
-                }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(w_empty + b);
+            if (b != eg) read_w(j);
         }
         const int r = 32 * q + lane;
         if (c0w < KW && r < N) {
