@@ -6,14 +6,14 @@
 //   k_node_bwd    recompute the node MLP from [a*, x], back-propagate dx_out:
 //                 da* (FP32) and dx_in = dx_out + d[x part]; dW of the node MLP
 //   halo          adjoint of Eq. 5c-5d = the same symmetric copy-sum on da*
-//   k_edge_bwd    recompute the edge MLP per receiver-aligned tile; the
+//   k_edge_bwd    (edge_bwd.cu) recompute the edge MLP per receiver-aligned tile; the
 //                 gradient of e' is de_out + da_i / d_ij (adjoint of Eq. 5b);
 //                 back-propagate to de_in = g + W1c^T dz1, write dz1 (the
 //                 gradient of the first pre-activation) per edge, sum it over
 //                 each receiver's edges into dP (FP32, fixed edge order); dW
 //   k_sender_sums, k_proj_bwd    dQ_j = sum of dz1 over the edges sent by j (sender CSR,
 //                 fixed order); dx_in += dP W1a + dQ W1b; dW1a, dW1b
-//   k_reduce      per-CTA weight-gradient partials summed in CTA order into dW
+//   k_reduce_grads    per-CTA weight-gradient partials summed in a fixed order into dW
 // No atomics anywhere: every sum has a fixed order, so results are bitwise
 // reproducible.
 //
@@ -513,7 +513,7 @@ struct CfgP {
     static constexpr int NT = 128 * CG;
 };
 
-// Two CTAs per SM up to H = 64; at H = 128 one (registers and shared memory).
+// One CTA per SM (the launch says why); the register bound leaves room for two up to H = 64.
 // The weight gradient [dW1a; dW1b] = [dP dQ]^T x is one M = 2H MMA up to
 // H = 64 and two M = 128 halves at H = 128.
 template <int H>
@@ -809,7 +809,9 @@ int proj_backward_h(const gnn_graph_dev& G, const gnn_mp_params& W, const float*
     int rc = persistent_grid(k_proj_bwd<H>, CfgP<H>::NT, P.total, pow2_cols(2 * H > 128 ? 3 * H : 2 * H),
                              (NR + 127) / 128, &grid);
     if (rc) return rc;
-    grid = std::min(grid, 2 * num_sms());
+    // One CTA per SM although two fit: the tensor core truncates its running sums, so the number of
+    // tiles one accumulator takes is part of dW1a's and dW1b's value (2 CTAs: 2e-5 apart at 6M rows).
+    grid = std::min(grid, num_sms());
     {
         ProfScope _ps(s, "k_proj_bwd");
         k_proj_bwd<H><<<grid, CfgP<H>::NT, P.total, s>>>(A);
