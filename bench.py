@@ -20,7 +20,7 @@ roofline  -- the whole step's algorithmic HBM bytes per unit of work (the
              against the measured HBM peak, beside the tensor-FLOP side; the
              slower side is the bound. roofline_kernel: the dominant kernel's
              event-timed launches against the bytes it moves as designed.
-fp32      -- the plain FP32 SIMT path against the fused BF16 path on the same
+fp32      -- the FP32 path against the fused BF16 path on the same
              graph (for the H=128 brick, on a 16^3-element p=7 sub-brick:
              the plain path's FP32 per-edge workspace does not fit the
              full graph).
@@ -278,7 +278,7 @@ def measured_traffic(workload: str, kernels: list, n_edges: int):
 
 
 def sgemm_flops_per_step(G, hidden: int, n_lin: int, layers: int) -> float:
-    """FP32 SIMT GEMM FLOPs of one plain-path step (forward, recompute, dgrad, wgrad)."""
+    """GEMM FLOPs of one step of the FP32 path's SIMT kernels, widths above 128 (forward, recompute, dgrad, wgrad)."""
     E, N, Hh = G.n_edges, G.n_rows, hidden
     def chain(rows, d0):
         dims = [d0] + [Hh] * n_lin
@@ -607,7 +607,7 @@ def measure_fp32_peak():
 
 
 def fp32_comparison(dev, wl: dict, part_full, steps: int, warmup: int, ms_bf16_full: float):
-    """The plain FP32 SIMT path against the fused BF16 path, same graph and step
+    """The FP32 path against the fused BF16 path, same graph and step
     (eager steps, median). For the H=128 brick the comparison graph is the
     16^3-element sub-brick of the same order and partition count."""
     import torch
@@ -620,7 +620,7 @@ def fp32_comparison(dev, wl: dict, part_full, steps: int, warmup: int, ms_bf16_f
         G, _, stack, dx, _, _ = build_problem(dev, prec, wl, part)
         run = prepare_timing(stack, dx, 2, graph=False)
         res[prec] = statistics.median(time_steps(run, steps, torch.cuda.current_stream()))
-        if prec == "fp32":   # the plain path's SIMT GEMMs against the measured FP32 FMA peak
+        if prec == "fp32":   # its SIMT GEMMs (widths above 128) against the measured FP32 FMA peak
             rep = _profiled(run, 1)
             n_lin = wl.get("nh", NH) + 2
             if "k_sgemm" in rep:
@@ -633,7 +633,7 @@ def fp32_comparison(dev, wl: dict, part_full, steps: int, warmup: int, ms_bf16_f
            "bf16_ms_per_step_same_graph": res["bf16"], "speedup_of_bf16": res["fp32"] / res["bf16"],
            "graph": "the benchmark graph" if sub_nel is None else
            f"{sub_nel}^3 elements p={wl['p']}, {wl['parts']} RCB sub-graphs ({L ** 3:,} nodes, {e_unpart:,} edges): "
-           "the plain path keeps FP32 per-edge activations ([E x 3H] input alone 105 GB at 32^3), which do not "
+           "the FP32 path keeps FP32 per-edge activations (35 GB per array at 32^3), which do not "
            "fit the full graph", "timing": "eager steps, median"}
     tf, sms = measure_fp32_peak()
     out["simt_peak"] = {"tflops": tf, "sm_count": sms,
