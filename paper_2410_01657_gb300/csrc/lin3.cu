@@ -7,11 +7,12 @@
 // FP32 by tcgen05.mma and the three left out (mid lo, lo mid, lo lo) are below
 // 2^-25 |x w|, of either sign. (Splitting by clearing bits costs the same but
 // makes every piece agree in sign with x: the parts left out then add up.)
-// The tensor core truncates its running sums, so a sum must not carry terms
-// far below it: the hi hi products have an accumulator of their own, the five
-// small ones one or two others, and the epilogue adds them up. Sums in tensor
-// memory run over at most 256 products per output (inputs) or one tile of rows
-// (weight gradients, continued in FP32 registers, rounding to nearest).
+// The tensor core truncates its running sums, so a sum must not carry terms far below it: a Linear's hi hi
+// products have an accumulator of their own up to width 64 (above, and in weight gradients of 65 to 128
+// inputs, the small products come first in a common one), the epilogue adds the accumulators up in FP32 and
+// gives back what truncation takes in the mean (kTruncation). Sums in tensor memory run over at most 256
+// products per output (inputs) or one tile of rows (weight gradients, continued in FP32 registers, rounding
+// to nearest).
 //
 // What bounds it: at width 64 a Linear moves 512 bytes per row for 49 kFLOP of
 // BF16 products, 96 FLOP per byte, far below the ridge: HBM, if the splitting
@@ -148,30 +149,39 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int la
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-// 16 columns of the lane's row: the hi hi sum plus the small products' sum (or sums, if three).
-__device__ __forceinline__ void load_sum16(uint32_t taddr, int NP, bool three, float* v) {
-    float u[16];
+// Accumulators of a row tile, NP columns each: what they hold, in the order in which they lie.
+enum Acc {
+    kAccAll,     // all six products
+    kAccHalves,  // all six products of the first | of the second half of the steps
+    kAccSmall,   // hi hi | the five small products
+    kAccThree    // hi hi | 2^-8 terms | 2^-16 terms
+};
+__host__ __device__ constexpr int acc_count(Acc acc) { return acc == kAccAll ? 1 : (acc == kAccThree ? 3 : 2); }
+
+// 16 columns of the lane's row: the accumulators' sum, with gain times the large products given back.
+template <Acc ACC>
+__device__ __forceinline__ void load_acc16(uint32_t taddr, int NP, float gain, float* v) {
+    float u[16], w[16];
     tmem_ld16(taddr, v);
-    tmem_ld16(taddr + NP, u);
-    if (three) {
-        float w[16];
-        tmem_ld16(taddr + 2 * NP, w);
-        tmem_ld_wait();
-#pragma unroll
-        for (int i = 0; i < 16; i += 2) {
-            const float2 z = __fadd2_rn(make_float2(u[i], u[i + 1]), make_float2(w[i], w[i + 1]));
-            u[i] = z.x;
-            u[i + 1] = z.y;
-        }
-    } else {
-        tmem_ld_wait();
-    }
+    if constexpr (ACC != kAccAll) tmem_ld16(taddr + NP, u);
+    if constexpr (ACC == kAccThree) tmem_ld16(taddr + 2 * NP, w);
+    tmem_ld_wait();
+    const float2 g = make_float2(gain, gain);
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
-        const float2 w = __fadd2_rn(make_float2(v[i], v[i + 1]), make_float2(u[i], u[i + 1]));
-        v[i] = w.x;
-        v[i + 1] = w.y;
+        const float2 a = make_float2(v[i], v[i + 1]);
+        float2 b = make_float2(u[i], u[i + 1]);
+        if constexpr (ACC == kAccThree) b = __fadd2_rn(b, make_float2(w[i], w[i + 1]));
+        const float2 r = ACC == kAccAll ? __fmul2_rn(g, a) : __ffma2_rn(g, ACC == kAccHalves ? __fadd2_rn(a, b) : a, b);
+        const float2 z = __fadd2_rn(a, r);
+        v[i] = z.x;
+        v[i + 1] = z.y;
     }
+}
+__device__ __forceinline__ void load_sum16(uint32_t taddr, int NP, Acc acc, float gain, float* v) {
+    if (acc == kAccThree) load_acc16<kAccThree>(taddr, NP, gain, v);
+    else if (acc == kAccHalves) load_acc16<kAccHalves>(taddr, NP, gain, v);
+    else load_acc16<kAccAll>(taddr, NP, gain, v);
 }
 
 // ELU (alpha 1) of two values: z above zero, e^z - 1 at and below it, by the
@@ -213,7 +223,27 @@ __device__ constexpr int kTermB[6] = {0, 2, 1, 0, 1, 0};
 // 2^-16 terms]. Per row tile at width 64: 1,650 cycles where the 24 narrow ones took 2,630. For a
 // weight gradient the terms of X are consecutive blocks of one MN-major operand, up to width 64
 // (1.0 -> 0.83 of the time at 64).
-__host__ __device__ inline bool three_sums(int NP) { return NP <= 80; }   // N = 3 NP <= 256
+//
+// Every step (16 of the contraction) cuts the running sum toward zero. Measured against 64 bits, 16 to 128
+// products: with normal or ELU operands a sum of n steps loses (n + 1) / 2 times 1.6e-8 to 1.9e-8 of its value
+// (up to 3.4e-8 where magnitudes are spread, nothing where all are alike). For one Linear that is below
+// FP32's rounding, but every row and layer loses in the same direction: on a network of width 64 (128) the
+// parameter gradients were 1.7 (3.5) times as far from 64 bits as with FP32 FMAs. So the epilogue of a Linear
+// gives the mean back (kTruncation: at most 4.5e-8 of a sum, below a unit in the last place), and above
+// width 64 the steps are halved between two accumulators. Networks of widths 8 to 128 against 64 bits, the
+// gradients' largest error over the FMAs': 0.57, their geometric mean 0.80. Weight gradients stay as
+// summed: their tiles are added in FP32, and their errors were below the FMAs' already.
+constexpr float kTruncation = 1.8e-8f;
+__host__ __device__ constexpr float gain_of(int steps) { return kTruncation * 0.5f * (float)(steps + 1); }
+
+// Two tiles' accumulators fit 512 columns. Up to width 64 three wide sums. Above, two of all six products
+// (smallest first): with two blocks a block each. With more blocks (two sources, up to width 80), where a
+// block's small products would follow another's large ones, three sums again. (Halves beside the small sums
+// up to width 64 too: errors 2 to 5 % smaller, a training step 2 %, a small call 6 % slower; not kept.)
+__host__ __device__ inline Acc acc_of(int NP, int KB, int nkb) {
+    if (NP <= 64 || nkb > 2) return kAccThree;
+    return nkb * KB > 16 ? kAccHalves : kAccAll;
+}
 
 // ------------------------------------------------------------------ shared memory
 
@@ -320,8 +350,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
     uint64_t* acc_full = full + 8;
     uint64_t* acc_empty = full + 10;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + P.tm);
-    const bool three = three_sums(NP);
-    const int ACC = (three ? 3 : 2) * NP;                       // columns of a tile's accumulators
+    const Acc acc = acc_of(NP, KB, nkb);
+    const int ACC = acc_count(acc) * NP;                        // columns of a tile's accumulators
     const uint32_t NCOLS = pow2_cols(2 * (uint32_t)ACC);        // two tiles
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -399,15 +429,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                     tc_fence_after();
                     const uint32_t ao = (uint32_t)st * 3 * P.aterm, wo = (uint32_t)b * 3 * P.wterm;
                     auto issue = [&](auto kb) {
-                        if (three) {
+                        constexpr int NS = decltype(kb)::value / 16;   // steps: one swizzle block, 32 bytes each
+                        const int half = nkb * NS / 2, s0 = b * NS;    // of the tile's steps; this block's first
+                        if (acc == kAccThree) {
                             const uint64_t wp = desc_step(w0, wo);
 #pragma unroll
                             for (int p = 0; p < 3; ++p) {
                                 const uint64_t ap = desc_step(a0, ao + p * P.aterm);
 #pragma unroll
-                                for (int k0 = 0; k0 < decltype(kb)::value; k0 += 16)   // one swizzle block, 32 bytes a step
-                                    mma_bf16_warp(lead, d + p * NP, desc_step(ap, k0 * 2), desc_step(wp, k0 * 2),
-                                                  p == 0 ? id3 : (p == 1 ? id2 : id), (b > 0 || p > 0 || k0 > 0) ? 1u : 0u);
+                                for (int k = 0; k < NS; ++k)
+                                    mma_bf16_warp(lead, d + p * NP, desc_step(ap, k * 32), desc_step(wp, k * 32),
+                                                  p == 0 ? id3 : (p == 1 ? id2 : id), (s0 + k > 0 || p > 0) ? 1u : 0u);
                             }
                             return;
                         }
@@ -416,9 +448,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                             const uint64_t ap = desc_step(a0, ao + kTermA[p] * P.aterm);
                             const uint64_t wp = desc_step(w0, wo + kTermB[p] * P.wterm);
 #pragma unroll
-                            for (int k0 = 0; k0 < decltype(kb)::value; k0 += 16)
-                                mma_bf16_warp(lead, p < 5 ? d + NP : d, desc_step(ap, k0 * 2), desc_step(wp, k0 * 2), id,
-                                         (b > 0 || (p > 0 && p < 5) || k0 > 0) ? 1u : 0u);
+                            for (int k = 0; k < NS; ++k) {
+                                const bool second = acc == kAccHalves && s0 + k >= half;
+                                mma_bf16_warp(lead, second ? d + NP : d, desc_step(ap, k * 32), desc_step(wp, k * 32), id,
+                                              (p > 0 || s0 + k > (second ? half : 0)) ? 1u : 0u);
+                            }
                         }
                     };
                     if (KB == 64) issue(Int<64>());
@@ -440,6 +474,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
         float* sums = reinterpret_cast<float*>(sm + P.sums) + ew * 2 * NP;
         const uint32_t tacc = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(eg * ACC);
         const int rs = lane >> 2, c4 = (lane & 3) * 4;
+        const int steps = (A.K[0] + 15) / 16 + (A.K[1] + 15) / 16;
+        const float gain = gain_of(acc == kAccHalves ? (steps + 1) / 2 : steps);
         constexpr bool kGather = MODE == kElu && OPS == kOpsGather, kEdge = MODE == kLnAdjoint && OPS == kOpsGather;
         bool ok = true;
         int j = 0;
@@ -504,7 +540,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                 float s4[4] = {0.f, 0.f, 0.f, 0.f};
                 for (int c0 = 0; c0 < N; c0 += 16) {
                     float v[16];
-                    load_sum16(tacc + c0, NP, three, v);
+                    load_sum16(tacc + c0, NP, acc, gain, v);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) s4[i & 3] += v[i] + sPar[c0 + i];   // padding columns are zero
                 }
@@ -512,7 +548,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                 float q4[4] = {0.f, 0.f, 0.f, 0.f};
                 for (int c0 = 0; c0 < N; c0 += 16) {
                     float v[16];
-                    load_sum16(tacc + c0, NP, three, v);
+                    load_sum16(tacc + c0, NP, acc, gain, v);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const float d = c0 + i < N ? v[i] + sPar[c0 + i] - mean : 0.f;
@@ -534,7 +570,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                         *reinterpret_cast<float4*>(stg + r * kStageLd + c4) = g[i];
                     }
                     float v[16];
-                    load_sum16(tacc + c0, NP, three, v);
+                    load_sum16(tacc + c0, NP, acc, gain, v);
                     __syncwarp();
 #pragma unroll
                     for (int i = 0; i < 16; i += 4) {
@@ -556,7 +592,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
             for (int c0 = 0; c0 < NP; c0 += 16) {
                 const int col = c0 + c4, nc = N - col;
                 float v[16];
-                load_sum16(tacc + c0, NP, three, v);
+                load_sum16(tacc + c0, NP, acc, gain, v);
                 if constexpr (MODE == kLayerNorm || MODE == kLnAdjoint) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] = (v[i] + sPar[c0 + i] - mean) * rstd;   // xhat
@@ -908,12 +944,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_wgrad3(const __grid_constant__
                 for (int i = 0; i < CW; i += 16) {
                     float v[16];
                     const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * SUMS * KP + c0 + i);
-                    if constexpr (SUMS == 3) {
-                        load_sum16(ta, KP, true, v);
-                    } else {
-                        tmem_ld16(ta, v);
-                        tmem_ld_wait();
-                    }
+                    load_acc16<SUMS == 3 ? kAccThree : kAccAll>(ta, KP, 0.f, v);
 #pragma unroll
                     for (int k = 0; k < 16; ++k) acc[i + k] += v[k];
                 }
@@ -1044,7 +1075,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
     float* sRed = reinterpret_cast<float*>(sm + P.red);
     // TMEM: dz' of two tiles, three sums each (at KW = 64 two: five MMAs a K-step), then dW, three
     // sums, of two tiles (at KW = 64 of one: the next tile's dz' is under way while it is read)
-    constexpr int ZS = KW <= 32 ? 3 : 2, WB = KW <= 32 ? 2 : 1;
+    constexpr Acc ZA = KW <= 32 ? kAccThree : kAccSmall;
+    constexpr int ZS = acc_count(ZA), WB = KW <= 32 ? 2 : 1;
     constexpr uint32_t WCOL = 2 * ZS * KW;
     constexpr uint32_t NCOLS = WCOL + WB * 3 * KW <= 256 ? 256 : 512;
     static_assert(WCOL + WB * 3 * KW <= 512, "tensor memory");
@@ -1190,6 +1222,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
 #pragma unroll
         for (int i = 0; i < CW; ++i) acc[i] = 0.f;
         bool ok = true;
+        const float zgain = gain_of((N + 15) / 16);
         // dW of tile j into the registers: by the tile's own group halfway through it, by the other
         // one after its tile before, at about the same time
         auto read_w = [&](int j) {
@@ -1201,7 +1234,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
 #pragma unroll
                 for (int i = 0; i < CW; i += 16) {
                     float v[16];
-                    load_sum16(tmem + lane_base + WCOL + (uint32_t)(wb * 3 * KW + c0w + i), KW, true, v);
+                    load_acc16<kAccThree>(tmem + lane_base + WCOL + (uint32_t)(wb * 3 * KW + c0w + i), KW, 0.f, v);
 #pragma unroll
                     for (int k = 0; k < 16; ++k) acc[i + k] += v[k];
                 }
@@ -1233,7 +1266,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
 #pragma unroll
                 for (int c0 = 0; c0 < KW; c0 += 16) {
                     float v[16];
-                    load_sum16(tacc + c0, KW, ZS == 3, v);
+                    load_acc16<ZA>(tacc + c0, KW, zgain, v);
 #pragma unroll
                     for (int i = 0; i < 16; i += 4)
                         *reinterpret_cast<float4*>(stg + lane * kStageLd + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
