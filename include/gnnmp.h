@@ -340,6 +340,8 @@ int gnn_mp_forward(const gnn_graph_dev* G, const gnn_mp_config* cfg, const gnn_m
  * parameter gradients into dW (same shapes as W, FP32) in a fixed order.
  * a_star: the forward's a_star_out, or NULL to recompute it. The halo adjoint
  * is the same copy-sum as the forward (the map a -> a* is symmetric).
+ * FP32: dx_in may be the buffer of x_in, dx_out or a_star, de_in that of e_in
+ * or de_out (same results).
  * BF16 at H = 128: the MLP adjoints run one Linear at a time over tiles of
  * 128 rows with the recomputed activations in workspace scratch, in chunks
  * of tiles; gnn_mp_workspace_size reports the size for the largest chunk,

@@ -290,7 +290,7 @@ __device__ __forceinline__ void lin_producer(const Args& A, const Smem& P, uint8
             for (int s = 0; s < 2; ++s)
                 if (A.K[s] && A.lda[s] == A.K[s]) prefetch_l2(A.A[s] + rn * A.lda[s], (uint32_t)(nr * A.K[s] * 4));
             if (A.add && A.ldadd == A.N) prefetch_l2(A.add + rn * A.N, (uint32_t)(nr * A.N * 4));
-            if (MODE == kLnAdjoint && A.g0) prefetch_l2(A.g0 + rn * A.N, (uint32_t)(nr * A.N * 4));
+            if ((MODE == kLnAdjoint || MODE == kAdd) && A.g0) prefetch_l2(A.g0 + rn * A.N, (uint32_t)(nr * A.N * 4));
         }
         const int left = (int)std::min<int64_t>(128, A.rows - (int64_t)t * 128);
         for (int b = 0; b < nkb; ++b) {
@@ -335,7 +335,7 @@ __device__ __forceinline__ void lin_producer(const Args& A, const Smem& P, uint8
 }
 
 // OPS: what an epilogue adds or needs of other rows: nothing, one row (add), or gathered rows
-// (P, Q of kElu; da, w of kLnAdjoint).
+// (P, Q of kElu; da, w of kLnAdjoint and kAdd).
 enum Ops { kOpsNone = 0, kOpsRow, kOpsGather };
 
 template <int MODE, int OPS, bool VEC>
@@ -476,7 +476,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
         const int rs = lane >> 2, c4 = (lane & 3) * 4;
         const int steps = (A.K[0] + 15) / 16 + (A.K[1] + 15) / 16;
         const float gain = gain_of(acc == kAccHalves ? (steps + 1) / 2 : steps);
-        constexpr bool kGather = MODE == kElu && OPS == kOpsGather, kEdge = MODE == kLnAdjoint && OPS == kOpsGather;
+        constexpr bool kGather = MODE == kElu && OPS == kOpsGather, kEdge = MODE != kElu && OPS == kOpsGather;
         bool ok = true;
         int j = 0;
         for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++j) {
@@ -495,38 +495,40 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                 if (kGather) sv[i] = A.snd[row[i]];
                 if (kEdge) wv[i] = A.w[row[i]];
             }
+            // the upstream gradient of one piece of the four rows, g0 or g0 + w da[recv]. It is formed wherever
+            // it is needed: a buffer for it would be the caller's gradient output, which may be one of the inputs
+            auto load_g = [&](int c0, float4* g) {
+                const int nc = N - (c0 + c4), col = VEC ? std::min(c0 + c4, N - 4) : c0 + c4;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) g[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (A.g0) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) g[i] = load4<VEC>(A.g0 + row[i] * N + col, VEC ? 4 : nc);
+                }
+                if constexpr (kEdge) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 d = load4<VEC>(A.da + (int64_t)rv[i] * N + col, VEC ? 4 : nc);
+                        g[i] = make_float4(fmaf(wv[i], d.x, g[i].x), fmaf(wv[i], d.y, g[i].y), fmaf(wv[i], d.z, g[i].z),
+                                           fmaf(wv[i], d.w, g[i].w));
+                    }
+                }
+            };
             // operands of one piece of the four rows
             auto load_ops = [&](int c0, float4* x, float4* y) {
                 const int nc = N - (c0 + c4), col = VEC ? std::min(c0 + c4, N - 4) : c0 + c4;
                 (void)y;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    if constexpr (kGather) {
-                        x[i] = load4<VEC>(A.P + (int64_t)rv[i] * A.ldpq + col, VEC ? 4 : nc);
-                        y[i] = load4<VEC>(A.Q + (int64_t)sv[i] * A.ldpq + col, VEC ? 4 : nc);
-                    } else if constexpr (MODE != kLnAdjoint && OPS == kOpsRow) {
-                        x[i] = load4<VEC>(A.add + row[i] * A.ldadd + col, VEC ? 4 : nc);
-                    }
-                }
-            };
-            // the upstream gradient of one piece of the four rows: formed (and, for edges, written by the
-            // same lane, perhaps over g0), then read again
-            auto load_g = [&](int c0, bool again, float4* g) {
-                const int nc = N - (c0 + c4), col = VEC ? std::min(c0 + c4, N - 4) : c0 + c4;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) g[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                const float* src = kEdge && again ? A.g_out : A.g0;
-                if (src) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) g[i] = load4<VEC>(src + row[i] * N + col, VEC ? 4 : nc);
-                }
-                if (kEdge && !again) {
+                if constexpr (MODE == kAdd && kEdge) {
+                    load_g(c0, x);
+                } else if constexpr (kGather) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const float4 d = load4<VEC>(A.da + (int64_t)rv[i] * N + col, VEC ? 4 : nc);
-                        g[i] = make_float4(g[i].x + wv[i] * d.x, g[i].y + wv[i] * d.y, g[i].z + wv[i] * d.z,
-                                           g[i].w + wv[i] * d.w);
+                        x[i] = load4<VEC>(A.P + (int64_t)rv[i] * A.ldpq + col, VEC ? 4 : nc);
+                        y[i] = load4<VEC>(A.Q + (int64_t)sv[i] * A.ldpq + col, VEC ? 4 : nc);
                     }
+                } else if constexpr (MODE != kLnAdjoint && OPS == kOpsRow) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) x[i] = load4<VEC>(A.add + row[i] * A.ldadd + col, VEC ? 4 : nc);
                 }
             };
             float4 x[4], y[4];
@@ -560,15 +562,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
             if constexpr (MODE == kLnAdjoint) {
                 // g, and its two row sums against gamma and gamma * xhat
                 for (int c0 = 0; c0 < N; c0 += 16) {
-                    const int col = c0 + c4, nc = N - col;
                     float4 g[4];
-                    load_g(c0, false, g);
+                    load_g(c0, g);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int r = 8 * i + rs;
-                        if (kEdge && r < nv) store4<VEC>(A.g_out + row[i] * N + col, nc, g[i]);
-                        *reinterpret_cast<float4*>(stg + r * kStageLd + c4) = g[i];
-                    }
+                    for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(stg + (8 * i + rs) * kStageLd + c4) = g[i];
                     float v[16];
                     load_sum16(tacc + c0, NP, acc, gain, v);
                     __syncwarp();
@@ -606,7 +603,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                     ga = *reinterpret_cast<const float4*>(sPar + NP + col);
                     be = *reinterpret_cast<const float4*>(sPar + 2 * NP + col);
                 }
-                if constexpr (MODE == kLnAdjoint) load_g(c0, true, x);
+                if constexpr (MODE == kLnAdjoint) load_g(c0, x);
                 __syncwarp();
                 float4 u[4];
 #pragma unroll
@@ -665,7 +662,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         u[i] = add4(u[i], b);
-                        if constexpr (OPS == kOpsRow) u[i] = add4(u[i], x[i]);
+                        if constexpr (OPS != kOpsNone) u[i] = add4(u[i], x[i]);
                     }
                 }
                 // the next piece's operands (an in-place sum reads other columns than it has written)
@@ -1383,7 +1380,7 @@ int run(Mode mode, Args a, cudaStream_t s, int* ctas) {
         if (a.K[i]) vec = vec && a.K[i] % 4 == 0 && a.lda[i] % 4 == 0 && aligned16(a.A[i]);
     vec = vec && (!a.add || (aligned16(a.add) && a.ldadd % 4 == 0));
     vec = vec && (!a.P || (aligned16(a.P) && aligned16(a.Q) && a.ldpq % 4 == 0));
-    vec = vec && aligned16(a.g0) && aligned16(a.da) && aligned16(a.g_out);
+    vec = vec && aligned16(a.g0) && aligned16(a.da);
     if (a.nsplit <= 0) a.nsplit = a.NP;
     const uint32_t smem = lin_smem(a.NP, a.KB, a.nkb[0] + a.nkb[1], a.stages).total;
     const int grid = (int)std::min<int64_t>(nt, std::min(kMaxCtas, fused::host::num_sms()));
@@ -1415,7 +1412,8 @@ int run(Mode mode, Args a, cudaStream_t s, int* ctas) {
             break;
         case kEluAdjoint: launch(Int<kEluAdjoint>(), one_row, "k_lin3_elu_adj"); break;
         case kAdd:
-            if (a.add) launch(Int<kAdd>(), one_row, "k_lin3_add");
+            if (a.da) launch(Int<kAdd>(), gather, "k_lin3_add");
+            else if (a.add) launch(Int<kAdd>(), one_row, "k_lin3_add");
             else launch(Int<kAdd>(), none, "k_lin3_add");
             break;
     }

@@ -18,7 +18,7 @@ enum Mode {
     kLayerNorm,   // out = res + gamma * xhat(acc + bias) + beta            (add = res, may be NULL)
     kLnAdjoint,   // out = dL/d(acc + bias) of the LayerNorm for the upstream g = g0, or g0 + w * da[recv]
     kEluAdjoint,  // out = acc * ELU'(z), add = h = ELU(z)
-    kAdd          // out = acc + bias + add
+    kAdd          // out = acc + bias + (add, or with da: g0 + w * da[recv])
 };
 
 struct Args {
@@ -44,7 +44,6 @@ struct Args {
     const float* g0;           // [rows x N] or NULL (zero)
     const float* da;           // [receivers x N] or NULL
     const float* w;            // [rows]
-    float* g_out;              // with da: [rows x N], g is also written here (may be g0)
     const float* gamma;
     const float* beta;
     float eps;

@@ -840,7 +840,7 @@ static int64_t tc_grad_floats(const gnn_mlp& P, int in, int sources) {
 
 // Adjoint of the last Linear's LayerNorm and of Linears n_lin-1 .. 1, from the
 // recomputed inputs hbuf[k]: returns dL/d(pre-activation 0) in *dz0 (one of
-// g0, g1). a: the upstream gradient's arguments (g0, da, w, recv, g_out);
+// g0, g1). a: the upstream gradient's arguments (g0, da, w, recv);
 // without LayerNorm the upstream gradient is dY itself.
 static int tc_chain_bwd(const gnn_mlp& P, const gnn_mlp& dP, int64_t rows, float* const* hbuf, float eps,
                         const lin3::Args& up, const float* dY, float* g0, float* g1, const float** dz0, GradSums& gs,
@@ -852,7 +852,7 @@ static int tc_chain_bwd(const gnn_mlp& P, const gnn_mlp& dP, int64_t rows, float
         lin3::Args a = lin_args(rows, hbuf[n - 1], P.dims[n - 1], P.dims[n - 1], P.W[n - 1], P.dims[n - 1], H,
                                 P.b[n - 1], g0, H);
         a.gamma = P.gamma; a.beta = P.beta; a.eps = eps;
-        a.g0 = up.g0; a.da = up.da; a.w = up.w; a.recv = up.recv; a.g_out = up.g_out;
+        a.g0 = up.g0; a.da = up.da; a.w = up.w; a.recv = up.recv;
         a.part = gs.part;
         int nz = 0;
         if ((rc = lin3::run(lin3::kLnAdjoint, a, s, &nz))) return rc;
@@ -884,7 +884,7 @@ static int tc_chain_bwd(const gnn_mlp& P, const gnn_mlp& dP, int64_t rows, float
 // ------------------------------------------------------------------ MP layer on the tensor cores
 
 struct TcBufs {
-    float* PQ;                    // [NR x 2H]: x W1a^T | x W1b^T
+    float* PQ;                    // [NR x 2H]: x W1a^T | x W1b^T; in the backward then dx_in's node part [NR x H]
     int32_t* recv;                // [E]
     float* hE[GNN_MAX_LIN];
     float* hN[GNN_MAX_LIN];
@@ -1013,6 +1013,8 @@ static int tc_mp_backward(const gnn_graph_dev& G, const gnn_mp_config& cfg, cons
     }
     if ((rc = tc_node_hidden(NR, H, W.node, a, x_in, b, s))) return rc;
 
+    // dx_in and de_in are written by the last launches alone, after x_in's and e_in's last use: each may be any
+    // of the inputs' buffers
     // node update adjoint (Eq. 5e)
     GradSums gs(b.part);
     const float* dz = nullptr;
@@ -1023,16 +1025,17 @@ static int tc_mp_backward(const gnn_graph_dev& G, const gnn_mp_config& cfg, cons
     if ((rc = gs.weight(NR, dz, H, x_in, H, H, dW.node.W[0] + H, 2 * H, nullptr, s))) return rc;
     lin3::Args l = dgrad_args(NR, dz, H, W.node.W[0], 2 * H, H, b.da, H);
     if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
-    l = dgrad_args(NR, dz, H, W.node.W[0] + H, 2 * H, H, dx_in, H);
+    float* dxn = b.PQ;
+    l = dgrad_args(NR, dz, H, W.node.W[0] + H, 2 * H, H, dxn, H);
     l.add = dx_out; l.ldadd = H;
     if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
     if ((rc = gs.flush(s))) return rc;
     // halo swap + sync adjoint (Eq. 5c-5d): the same symmetric copy-sum
     if (cfg.halo_mode == GNN_HALO_SYNC && (rc = halo(G, b.da, H, s))) return rc;
 
-    // edge update adjoint (Eq. 5a): the gradient of e' is de_out + w da_i (adjoint of Eq. 5b), kept in de_in
+    // edge update adjoint (Eq. 5a): the gradient of e' is de_out + w da_i (adjoint of Eq. 5b)
     up = lin3::Args{};
-    up.g0 = de_out; up.da = b.da; up.w = G.edge_w; up.recv = b.recv; up.g_out = de_in;
+    up.g0 = de_out; up.da = b.da; up.w = G.edge_w; up.recv = b.recv;
     if ((rc = tc_chain_bwd(W.edge, dW.edge, E, b.hE, cfg.ln_eps, up, nullptr, b.g0, b.g1, &dz, gs, s))) return rc;
     if (E && (rc = gs.weight(E, dz, H, e_in, H, H, dW.edge.W[0] + 2 * H, 3 * H, dW.edge.b[0], s))) return rc;
     if (NR) {
@@ -1046,17 +1049,19 @@ static int tc_mp_backward(const gnn_graph_dev& G, const gnn_mp_config& cfg, cons
         GNN_LAUNCH_CHECK("k_node_sums");
     }
     l = dgrad_args(E, dz, H, W.edge.W[0] + 2 * H, 3 * H, H, de_in, H);
-    l.add = de_in; l.ldadd = H;
+    l.g0 = up.g0; l.da = up.da; l.w = up.w; l.recv = up.recv;
     if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
     if ((rc = gs.weight(NR, b.dP, H, x_in, H, H, dW.edge.W[0], 3 * H, nullptr, s))) return rc;
     if ((rc = gs.weight(NR, b.dQ, H, x_in, H, H, dW.edge.W[0] + H, 3 * H, nullptr, s))) return rc;
     l = dgrad_args(NR, b.dP, H, W.edge.W[0], 3 * H, H, dx_in, H);
-    l.add = dx_in; l.ldadd = H;
+    l.add = dxn; l.ldadd = H;
     if (lin3::fits(H, H, 2)) {
         l.A[1] = b.dQ; l.lda[1] = H; l.K[1] = H; l.W[1] = W.edge.W[0] + H;
         if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
     } else {
+        l.out = dxn;
         if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
+        l.out = dx_in;
         l.A[0] = b.dQ; l.W[0] = W.edge.W[0] + H;
         if ((rc = lin3::run(lin3::kAdd, l, s))) return rc;
     }
