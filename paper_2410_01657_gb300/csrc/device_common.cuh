@@ -44,6 +44,22 @@ __device__ __forceinline__ float from_f32<float>(float v) { return v; }
 template <>
 __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
+// True unless the two [rows x cols] destinations (row strides ld) are certainly apart: different ranges, or
+// different columns of rows of one stride. One launch adds only to destinations that are apart; a
+// parameter tied to another has one gradient buffer for both.
+struct Dest {
+    const float* p;
+    int64_t ld;
+    int rows, cols;
+};
+inline bool may_overlap(const Dest& a, const Dest& b) {
+    const float *ae = a.p + (a.rows - 1) * a.ld + a.cols, *be = b.p + (b.rows - 1) * b.ld + b.cols;
+    if (ae <= b.p || be <= a.p) return false;
+    if (a.ld != b.ld || a.ld <= 0) return true;
+    const int64_t off = (((b.p - a.p) % a.ld) + a.ld) % a.ld;   // b's first column in a's rows
+    return !(off >= a.cols && off + b.cols <= a.ld);
+}
+
 inline int cuda_fail(cudaError_t e, const char* what) {
     return set_error(GNN_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }

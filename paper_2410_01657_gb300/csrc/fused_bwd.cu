@@ -715,20 +715,29 @@ __global__ void __launch_bounds__(256) k_reduce_grads(const __grid_constant__ Re
 int reduce_grads(RedSeg* segs, int n, cudaStream_t s) {
     RedArgs A{};
     GNN_REQUIRE(n <= MAX_SEGS, GNN_EUNSUPPORTED, "reduce_grads: too many segments");
+    auto flush = [&]() -> int {
+        const int blocks = A.blk[A.n_seg];
+        if (blocks == 0) return GNN_OK;
+        {
+            ProfScope _ps(s, "k_reduce_grads");
+            k_reduce_grads<<<blocks, 256, 0, s>>>(A);
+        }
+        A.n_seg = 0;
+        GNN_LAUNCH_CHECK("k_reduce_grads");
+        return GNN_OK;
+    };
+    auto dest = [](const RedSeg& g) { return Dest{g.dst, g.dst_ld, g.rows, g.cols}; };
+    int rc;
     for (int i = 0; i < n; ++i) {
         if (segs[i].n_cta <= 0) continue;
+        bool apart = true;
+        for (int k = 0; k < A.n_seg; ++k) apart = apart && !may_overlap(dest(A.seg[k]), dest(segs[i]));
+        if (!apart && (rc = flush())) return rc;
         A.seg[A.n_seg] = segs[i];
         A.blk[A.n_seg + 1] = A.blk[A.n_seg] + (segs[i].rows * segs[i].cols + 31) / 32;
         ++A.n_seg;
     }
-    const int blocks = A.blk[A.n_seg];
-    if (blocks == 0) return GNN_OK;
-    {
-        ProfScope _ps(s, "k_reduce_grads");
-        k_reduce_grads<<<blocks, 256, 0, s>>>(A);
-    }
-    GNN_LAUNCH_CHECK("k_reduce_grads");
-    return GNN_OK;
+    return flush();
 }
 
 int reduce_grads(RedSeg* segs, int n, const float* part, int64_t pstride, int n_cta, cudaStream_t s) {

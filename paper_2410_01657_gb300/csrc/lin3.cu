@@ -1507,21 +1507,29 @@ int chain(int64_t rows, const float* G, int N, const float* H, int K, const floa
 int reduce(const Sum* sums, int n, cudaStream_t s) {
     RedArgs a{};
     int blocks = 0;
+    auto flush = [&]() -> int {
+        if (blocks == 0) return GNN_OK;
+        a.first[a.n] = blocks;
+        {
+            ProfScope _ps(s, "k_reduce3");
+            k_reduce3<<<blocks, 256, 0, s>>>(a);
+        }
+        a.n = blocks = 0;
+        GNN_LAUNCH_CHECK("k_reduce3");
+        return GNN_OK;
+    };
+    auto dest = [](const Sum& q) { return Dest{q.dst, q.ldd, q.N, q.K}; };
+    int rc;
     for (int i = 0; i < n; ++i) {
         if (sums[i].nz == 0 || !sums[i].dst) continue;
-        GNN_REQUIRE(a.n < kMaxReduce, GNN_EUNSUPPORTED, "lin3: too many sums");
+        bool apart = a.n < kMaxReduce;
+        for (int k = 0; k < a.n; ++k) apart = apart && !may_overlap(dest(a.s[k]), dest(sums[i]));
+        if (!apart && (rc = flush())) return rc;
         a.s[a.n] = sums[i];
         a.first[a.n++] = blocks;
         blocks += (sums[i].N * sums[i].K + 31) / 32;
     }
-    a.first[a.n] = blocks;
-    if (blocks == 0) return GNN_OK;
-    {
-        ProfScope _ps(s, "k_reduce3");
-        k_reduce3<<<blocks, 256, 0, s>>>(a);
-    }
-    GNN_LAUNCH_CHECK("k_reduce3");
-    return GNN_OK;
+    return flush();
 }
 
 }  // namespace lin3

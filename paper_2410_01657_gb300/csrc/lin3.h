@@ -69,7 +69,8 @@ bool chain_fits(int N, int K);
 int chain(int64_t rows, const float* G, int N, const float* H, int K, const float* W, float* out, bool db, float* part,
           cudaStream_t s, int* ctas);
 
-// dst[n * ldd + k] += sum over z of part[z * stride + n * K + k], z ascending per lane.
+// dst[n * ldd + k] += sum over z of part[z * stride + n * K + k], z ascending per lane. One launch, and another
+// wherever a destination may overlap an earlier one.
 struct Sum {
     const float* part;
     int64_t stride;
