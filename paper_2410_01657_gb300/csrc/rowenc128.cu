@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(kW0NT) k_rowenc_w0(W0Args A) {
 template <int KQ>
 __global__ void __launch_bounds__(kW0NT) k_rowenc_w0_rows(const __grid_constant__ W0Args A) {
     constexpr int CPT = 8 / KQ, TPR = kH / CPT, RPB = kW0NT / TPR, U = 4;
-    __shared__ float red[kH * 4 * KQ];
+    __shared__ __align__(16) float red[kH * 4 * KQ];
     const int tid = threadIdx.x, c0 = (tid % TPR) * CPT, rg = tid / TPR, K0 = A.K0;
     const int64_t r_begin = A.t0 * 128, r_end = A.t1 * 128 < A.n_rows ? A.t1 * 128 : A.n_rows;
     const int64_t step = (int64_t)gridDim.x * RPB;
