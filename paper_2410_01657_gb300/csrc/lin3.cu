@@ -2,7 +2,9 @@
 //
 // An FP32 number has 24 significant bits, so it is exactly the sum of three
 // BF16 numbers of 8 bits each: hi = x rounded to BF16, mid = x - hi rounded,
-// lo = the rest (both differences are exact). A product x w is then the sum of
+// lo = the rest (both differences are exact; numbers are scaled first, see kUp,
+// so that this holds for the smallest ones, and from 2^104 on and for infinities
+// FP32 FMAs take over). A product x w is then the sum of
 // nine BF16 products, each exact in FP32; the six largest are accumulated in
 // FP32 by tcgen05.mma and the three left out (mid lo, lo mid, lo lo) are below
 // 2^-25 |x w|, of either sign. (Splitting by clearing bits costs the same but
@@ -70,12 +72,35 @@ __host__ __device__ inline uint32_t pow2_cols(uint32_t n) {
 
 // ------------------------------------------------------------------ device helpers
 
-// Eight FP32 values as three BF16 octets whose sum they are.
+// The ends of the range. Streamed operands are split at 2^24 of their size, so that the last bit of the
+// smallest FP32 number is a normal BF16 number, and weights at 2^-24, which leaves a Linear's sums as they
+// are; a weight gradient's two streamed operands leave 2^48, taken off where its tiles are added. No bit of
+// a sum in the middle of the range changes by it.
+//
+// The other end cannot be split. From 2^104 on, and for infinities, hi is infinite, and every sum that the
+// number is in is a NaN: all columns of its row. So the epilogue looks at one column of each row (LayerNorm:
+// at the mean), and a tile in which that is not finite is begun again after a function out of line has
+// replaced the sums that are not finite by FP32 FMAs. Weights are looked at when they are split, eight
+// at a time: one above 2^16 (below, a sum that overflows has a number above 2^104 in it), or eight
+// below 2^-80, whose pieces lose bits and one of which is made a NaN, send every tile of the block there. A
+// weight gradient's sums are looked at when the block is done. A training step at width 64 takes 9.58 -> 9.69 ms
+// with it, a 4-cube forward 77.5 -> 81.4 us (checking all sums in the epilogue, or the numbers in the
+// producers, cost 9 and 4 % more of the step).
+constexpr float kUp = 16777216.f, kDown = 1.f / 16777216.f, kUnscale = kDown * kDown;
+constexpr float kBigWeight = 65536.f;                     // 2^16
+constexpr float kTinyWeights = 8.271806125530277e-25f;    // 2^-80
+
+__device__ __forceinline__ bool finite(float v) { return fabsf(v) <= 3.402823466e38f; }
+
+// Eight FP32 values times 2^24 (DOWN: 2^-24) as three BF16 octets whose sum they are.
+template <bool DOWN = false>
 __device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& mid, uint4& lo) {
     uint32_t h[4], m[4], l[4];
+    constexpr float kS = DOWN ? kDown : kUp;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        float a = v[2 * i], b = v[2 * i + 1], x, y;
+        const float2 t = __fmul2_rn(make_float2(v[2 * i], v[2 * i + 1]), make_float2(kS, kS));
+        float a = t.x, b = t.y, x, y;
         h[i] = pack_bf16x2(a, b);
         unpack_bf16x2(h[i], x, y);
         a -= x;
@@ -87,6 +112,15 @@ __device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& mid, ui
     hi = make_uint4(h[0], h[1], h[2], h[3]);
     mid = make_uint4(m[0], m[1], m[2], m[3]);
     lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// Eight weights of a row: true if they are special.
+__device__ __forceinline__ bool check_weights(float* v) {
+    const float m = fmaxf(fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3]))),
+                          fmaxf(fmaxf(fabsf(v[4]), fabsf(v[5])), fmaxf(fabsf(v[6]), fabsf(v[7]))));
+    const bool tiny = m > 0.f && m < kTinyWeights;
+    if (tiny) v[0] = __uint_as_float(0x7fffffffu);
+    return tiny || !(m <= kBigWeight);
 }
 
 // Up to n (may be <= 0) of the 8 values at p, the rest zero. VEC: p is 16-byte
@@ -149,6 +183,19 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int la
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
+// 16 values into 16 consecutive TMEM columns of this thread's lane.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
+    uint32_t r[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(v[i]);
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
+            taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+
 // Accumulators of a row tile, NP columns each: what they hold, in the order in which they lie.
 enum Acc {
     kAccAll,     // all six products
@@ -182,6 +229,73 @@ __device__ __forceinline__ void load_sum16(uint32_t taddr, int NP, Acc acc, floa
     if (acc == kAccThree) load_acc16<kAccThree>(taddr, NP, gain, v);
     else if (acc == kAccHalves) load_acc16<kAccHalves>(taddr, NP, gain, v);
     else load_acc16<kAccAll>(taddr, NP, gain, v);
+}
+
+// Sums that are not finite, by FP32 FMAs from global memory, in order.
+struct LinSum {   // of a row of a Linear
+    const Args& A;
+    int64_t row;
+    __device__ float operator()(int n) const {
+        const int64_t off = n >= A.nsplit ? A.noff + (int64_t)(n - A.nsplit) * A.sn : (int64_t)n * A.sn;
+        float t = 0.f;
+        for (int s = 0; s < 2 && n < A.N; ++s) {
+#pragma unroll 8
+            for (int k = 0; k < A.K[s]; ++k) t = fmaf(A.A[s][row * A.lda[s] + k], A.W[s][off + k * A.sk], t);
+        }
+        return t;
+    }
+};
+struct RowSum {   // sum over j < n of a[j] b[j ld + i], zero for i >= ld
+    const float* a;
+    const float* b;
+    int n, ld;
+    __device__ float operator()(int i) const {
+        float t = 0.f;
+        if (i >= ld) return t;
+#pragma unroll 8
+        for (int j = 0; j < n; ++j) t = fmaf(a[j], b[(int64_t)j * ld + i], t);
+        return t;
+    }
+};
+
+// The accumulators (NP columns of the warp's rows) with every sum that is not finite replaced.
+template <class F>
+__device__ __noinline__ void patch_sums(const F& exact, bool mine, uint32_t taddr, int NP, Acc acc, float gain) {
+    for (int c0 = 0; c0 < NP; c0 += 16) {
+        float v[16], w[16];
+        uint32_t bad = 0;
+        load_sum16(taddr + c0, NP, acc, gain, v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) bad |= (mine && !finite(v[i])) ? 1u << i : 0u;
+        if (!__any_sync(0xffffffffu, bad != 0)) continue;
+        for (int i = 0; i < 16; ++i) {
+            const float t = (bad >> i) & 1u ? exact(c0 + i) : 0.f;
+            w[i] = finite(t) ? fmaf(-gain, t, t) : t;   // (the gain is given back when it is read)
+        }
+        __syncwarp();
+        for (int a = 0; a < acc_count(acc); ++a) {
+            tmem_ld16(taddr + (uint32_t)(a * NP + c0), v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if ((bad >> i) & 1u) v[i] = a == 0 ? w[i] : 0.f;
+            tmem_st16(taddr + (uint32_t)(a * NP + c0), v);
+        }
+        tmem_st_wait();
+    }
+}
+// sum over the block's row tiles (RT rows each) of G[r ldg] X[r ldx]
+__device__ __noinline__ float dw_sum(const float* G, int64_t ldg, const float* X, int64_t ldx, int64_t rows, int n_tiles,
+                                     int RT) {
+    float s = 0.f;
+    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+        const int64_t r1 = std::min<int64_t>(rows, (int64_t)(t + 1) * RT);
+        float a = 0.f;
+#pragma unroll 8
+        for (int64_t r = (int64_t)t * RT; r < r1; ++r) a = fmaf(G[r * ldg], X[r * ldx], a);
+        s += a;
+    }
+    return s;
 }
 
 // ELU (alpha 1) of two values: z above zero, e^z - 1 at and below it, by the
@@ -370,6 +484,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
         }
         fence_mbar_init();
     }
+    bool special_w = false;
     {   // the weights, split, for the block's lifetime
         const int upr = KB / 8, per = NP * upr;
         for (int i = tid; i < nkb * per; i += kThreads) {
@@ -381,8 +496,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
             float v[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) v[j] = (n < N && k0 + j < A.K[s]) ? __ldg(w + (k0 + j) * A.sk) : 0.f;
+            special_w |= check_weights(v);
             uint4 t[3];
-            split8(v, t[0], t[1], t[2]);
+            split8<true>(v, t[0], t[1], t[2]);
             const uint32_t off = tile_off(n, k8, NP, S);
 #pragma unroll
             for (int j = 0; j < 3; ++j) *reinterpret_cast<uint4*>(sm + P.w + (b * 3 + j) * P.wterm + off) = t[j];
@@ -401,7 +517,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
     }
     fence_proxy_async();
     tc_fence_before();
-    __syncthreads();
+    const float spoil = __syncthreads_or(special_w) ? __uint_as_float(0x7fffffffu) : 0.f;   // not finite if special
     tc_fence_after();
     const uint32_t tmem = *tslot;
 
@@ -478,9 +594,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
         const float gain = gain_of(acc == kAccHalves ? (steps + 1) / 2 : steps);
         constexpr bool kGather = MODE == kElu && OPS == kOpsGather, kEdge = MODE != kElu && OPS == kOpsGather;
         bool ok = true;
-        int j = 0;
-        for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++j) {
-            if ((j & 1) != eg) continue;
+        int j = 0, t = blockIdx.x;
+        // a tile that turns out to be special (nothing of it has been written by then) is patched and begun again
+        bool patched = false;
+        auto next = [&] {
+            t += gridDim.x;
+            ++j;
+            patched = false;
+        };
+        while (t < A.n_tiles && ok) {
+            if ((j & 1) != eg) {
+                next();
+                continue;
+            }
             const int64_t rb = (int64_t)t * 128 + 32 * q;
             const int nv = (int)std::min<int64_t>(32, std::max<int64_t>(0, A.rows - rb));
             // this lane's rows (clamped to the last one: loads need no test, stores have it) and their
@@ -536,6 +662,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
             ok = warp_wait(acc_full + eg, (uint32_t)(j >> 1) & 1u, lane);
             if (!ok) break;
             tc_fence_after();
+            auto special = [&](float v) {
+                if (patched || !__any_sync(0xffffffffu, lane < nv && !finite(v + spoil))) return false;
+                patch_sums(LinSum{A, lane < nv ? rb + lane : 0}, lane < nv, tacc, NP, acc, gain);
+                return patched = true;
+            };
             float mean = 0.f, rstd = 0.f, m1 = 0.f, m2 = 0.f;
             if constexpr (MODE == kLayerNorm || MODE == kLnAdjoint) {
                 // row statistics: the lane's row, two passes over the accumulator
@@ -547,6 +678,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                     for (int i = 0; i < 16; ++i) s4[i & 3] += v[i] + sPar[c0 + i];   // padding columns are zero
                 }
                 mean = ((s4[0] + s4[1]) + (s4[2] + s4[3])) / N;
+                if (special(mean)) continue;
                 float q4[4] = {0.f, 0.f, 0.f, 0.f};
                 for (int c0 = 0; c0 < N; c0 += 16) {
                     float v[16];
@@ -586,10 +718,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                 m1 /= N;
                 m2 /= N;
             }
+            bool again = false;
             for (int c0 = 0; c0 < NP; c0 += 16) {
                 const int col = c0 + c4, nc = N - col;
                 float v[16];
                 load_sum16(tacc + c0, NP, acc, gain, v);
+                if (MODE != kLayerNorm && MODE != kLnAdjoint && c0 == 0 && (again = special(v[0]))) break;
                 if constexpr (MODE == kLayerNorm || MODE == kLnAdjoint) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] = (v[i] + sPar[c0 + i] - mean) * rstd;   // xhat
@@ -679,9 +813,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_lin3(const __grid_constant__ Ar
                     if (8 * i + rs < nv) store4<VEC>(A.out + row[i] * A.ldo + col, nc, u[i]);
                 __syncwarp();
             }
+            if (again) continue;
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(acc_empty + eg);
+            next();
         }
     }
     tc_fence_before();
@@ -943,7 +1079,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_wgrad3(const __grid_constant__
                     const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * SUMS * KP + c0 + i);
                     load_acc16<SUMS == 3 ? kAccThree : kAccAll>(ta, KP, 0.f, v);
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) acc[i + k] += v[k];
+                    for (int k = 0; k < 16; ++k) acc[i + k] = fmaf(v[k], kUnscale, acc[i + k]);
                 }
             }
             tc_fence_before();
@@ -953,8 +1089,12 @@ __global__ void __launch_bounds__(kWThreads, 1) k_wgrad3(const __grid_constant__
         const int r = 32 * q + lane;
         if (work && r < N) {
 #pragma unroll
-            for (int i = 0; i < CW; ++i)
-                if (c0 + i < K) part[(int64_t)r * K + c0 + i] = acc[i];
+            for (int i = 0; i < CW; ++i) {
+                if (c0 + i >= K) continue;
+                float* o = part + (int64_t)r * K + c0 + i;
+                *o = acc[i];
+                if (!finite(acc[i])) *o = dw_sum(A.G + r, A.ldg, A.X + c0 + i, A.ldx, A.rows, A.n_tiles, RT);
+            }
         }
     }
     tc_fence_before();
@@ -1097,21 +1237,23 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
         mbar_init(empty_h, 1);
         fence_mbar_init();
     }
+    bool special_w = false;
     // W^T as the [KW x NW] K-major operand of dz W: row k, column n
     for (int i = tid; i < KW * (NW / 8); i += kThreads) {
         const int k = i / (NW / 8), n8 = (i % (NW / 8)) * 8;
         float v[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) v[j] = (k < K && n8 + j < N) ? __ldg(A.W + (int64_t)(n8 + j) * K + k) : 0.f;
+        special_w |= check_weights(v);
         uint4 t[3];
-        split8(v, t[0], t[1], t[2]);
+        split8<true>(v, t[0], t[1], t[2]);
         const uint32_t off = tile_off(k, n8, KW, Sg);
 #pragma unroll
         for (int j = 0; j < 3; ++j) *reinterpret_cast<uint4*>(sm + P.w + j * P.wterm + off) = t[j];
     }
     fence_proxy_async();
     tc_fence_before();
-    __syncthreads();
+    const float spoil = __syncthreads_or(special_w) ? __uint_as_float(0x7fffffffu) : 0.f;   // not finite if special
     tc_fence_after();
     const uint32_t tmem = *tslot;
     float* part = A.part + (int64_t)blockIdx.x * (N * K + (A.db ? N : 0));
@@ -1233,15 +1375,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
                     float v[16];
                     load_acc16<kAccThree>(tmem + lane_base + WCOL + (uint32_t)(wb * 3 * KW + c0w + i), KW, 0.f, v);
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) acc[i + k] += v[k];
+                    for (int k = 0; k < 16; ++k) acc[i + k] = fmaf(v[k], kUnscale, acc[i + k]);
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(w_empty + wb);
         };
-        int j = 0;
-        for (int t = blockIdx.x; t < A.n_tiles && ok; t += gridDim.x, ++j) {
+        int j = 0, t = blockIdx.x;
+        bool patched = false;   // as in k_lin3; a special tile is begun again before its dW is read
+        while (t < A.n_tiles && ok) {
             const int b = j & 1;
             if (b == eg) {   // this group's tile: dz' = acc ELU'(h)
                 const int64_t rb = (int64_t)t * 128 + 32 * q;
@@ -1260,10 +1403,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t tacc = tmem + lane_base + (uint32_t)(b * ZS * KW);
+                bool again = false;
 #pragma unroll
                 for (int c0 = 0; c0 < KW; c0 += 16) {
                     float v[16];
                     load_acc16<ZA>(tacc + c0, KW, zgain, v);
+                    if (c0 == 0 && !patched && __any_sync(0xffffffffu, lane < nv && !finite(v[0] + spoil))) {
+                        patch_sums(RowSum{A.G + (lane < nv ? rb + lane : 0) * N, A.W, N, K}, lane < nv, tacc, KW, ZA, zgain);
+                        again = patched = true;
+                        break;
+                    }
 #pragma unroll
                     for (int i = 0; i < 16; i += 4)
                         *reinterpret_cast<float4*>(stg + lane * kStageLd + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
@@ -1282,17 +1431,25 @@ __global__ void __launch_bounds__(kThreads, 1) k_chain3(const __grid_constant__ 
                     __syncwarp();
                     if (c0 == (KW == 64 ? 16 : 0)) read_w(j);
                 }
+                if (again) continue;
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(acc_empty + b);
             }
             if (b != eg) read_w(j);
+            t += gridDim.x;
+            ++j;
+            patched = false;
         }
         const int r = 32 * q + lane;
         if (c0w < KW && r < N) {
 #pragma unroll
-            for (int i = 0; i < CW; ++i)
-                if (c0w + i < K) part[(int64_t)r * K + c0w + i] = acc[i];
+            for (int i = 0; i < CW; ++i) {
+                if (c0w + i >= K) continue;
+                float* o = part + (int64_t)r * K + c0w + i;
+                *o = acc[i];
+                if (!finite(acc[i])) *o = dw_sum(A.G + r, N, A.H + c0w + i, K, A.rows, A.n_tiles, 128);
+            }
         }
     }
     tc_fence_before();
