@@ -49,12 +49,19 @@ def n_mlp_tensors(dims, has_ln: bool) -> int:
 
 
 def zero_grads(tensors) -> tuple:
-    """(flat, views): zeroed gradient buffers shaped like ``tensors``, pieces of one
+    """(flat, pieces): zeroed gradient buffers shaped like ``tensors``, pieces of one
     flat allocation, so that zeroing them is one launch instead of one per tensor
     (a layer has 20 and more: on small graphs those launches took longer than
-    the layer's kernels)."""
-    flat = torch.zeros(sum(t.numel() for t in tensors), dtype=torch.float32, device=tensors[0].device)
-    return flat, [v.view(t.shape) for v, t in zip(flat.split([t.numel() for t in tensors]), tensors)]
+    the layer's kernels). The pieces are tensors on that storage, not views: each
+    has its own version counter, as gradients of separate allocations have. They
+    start 256 bytes apart or at multiples of it."""
+    sizes = [(t.numel() + 63) // 64 * 64 for t in tensors]
+    flat = torch.zeros(sum(sizes), dtype=torch.float32, device=tensors[0].device)
+    pieces, at = [], 0
+    for t, n in zip(tensors, sizes):
+        pieces.append(flat.new_empty(0).set_(flat.untyped_storage(), at, t.shape))
+        at += n
+    return flat, pieces
 
 
 def mp_config(hidden: int, precision: str, halo: bool = True, ln_eps: float = 1e-5, flags: int = 0):
