@@ -783,11 +783,12 @@ BwdWs carve_bwd(void* ws, const gnn_graph_dev& G, int H, int Le, int Ln, bool ne
     w.da = (float*)take((size_t)NR * H * 4);
     w.dP = (float*)take((size_t)NR * H * 4);
     w.dz1 = (__nv_bfloat16*)take((size_t)E * H * 2);
-    // per-CTA weight-gradient partials: one CTA per SM for the edge and node kernels, up to two per
-    // SM for the projection kernel; apart, so that one launch sums them all
-    w.part_node = (float*)take((size_t)ncta * node_pstride(H, Ln) * 4);
+    // per-CTA weight-gradient partials, apart, so that one launch sums them all: at most one CTA per SM and
+    // row tile (the edge kernel's tiles may change after the workspace has been sized)
+    const int64_t nrow = std::min(ncta, (NR + 127) / 128);
+    w.part_node = (float*)take((size_t)nrow * node_pstride(H, Ln) * 4);
     w.part_edge = (float*)take((size_t)ncta * edge_pstride(H, Le) * 4);
-    w.part_proj = (float*)take((size_t)2 * ncta * proj_pstride(H) * 4);
+    w.part_proj = (float*)take((size_t)nrow * proj_pstride(H) * 4);
     w.bytes = off + 256;
     return w;
 }

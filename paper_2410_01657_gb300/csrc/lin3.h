@@ -9,7 +9,7 @@ namespace gnn {
 namespace lin3 {
 
 constexpr int kMaxWidth = 128;   // widest N and K of one launch (per source)
-constexpr int kMaxCtas = 160;    // most CTAs of a launch: sizes the per-CTA partial sums
+constexpr int kMaxCtas = 160;    // most CTAs of a launch
 constexpr int kMaxReduce = 24;   // most sums of one reduce launch
 
 // What happens to a row tile's products acc = sum_s A_s W_s^T on their way out.
@@ -61,7 +61,9 @@ bool fits(int N, int K, int sources);
 // of sum_r G[r][n] ([N] behind it) into part; *ctas receives their number.
 int wgrad(int64_t rows, const float* G, int64_t ldg, int N, const float* X, int64_t ldx, int K, bool db, float* part,
           cudaStream_t s, int* ctas);
-inline int64_t wgrad_floats(int N, int K) { return (int64_t)kMaxCtas * (N * K + N); }
+// Most CTAs of a launch over `rows` rows (a row tile has 64 or 128): sizes the per-CTA partial sums.
+inline int64_t max_ctas(int64_t rows) { return rows + 63 < (int64_t)kMaxCtas * 64 ? (rows + 63) / 64 : kMaxCtas; }
+inline int64_t wgrad_floats(int64_t rows, int N, int K) { return max_ctas(rows) * (N * K + N); }
 
 // out [rows x K] = (G W) ELU'(H) and the partials of wgrad(G, H) in one pass
 // (G [rows x N], H = ELU outputs [rows x K], W [N x K], all dense).

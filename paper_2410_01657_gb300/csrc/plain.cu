@@ -816,7 +816,7 @@ struct GradSums {
         const int64_t stride = (int64_t)N * K + (db ? N : 0);
         s[n++] = {part, stride, nz, N, K, dW, ldw};
         if (db) s[n++] = {part + (int64_t)N * K, stride, nz, 1, N, db, N};
-        part += lin3::wgrad_floats(N, K);
+        part += lin3::wgrad_floats(rows, N, K);
         return GNN_OK;
     }
     // the same with X = ELU outputs, and out = (G W) ELU'(X), in one pass
@@ -828,13 +828,15 @@ struct GradSums {
         const int64_t stride = (int64_t)N * K + N;
         s[n++] = {part, stride, nz, N, K, dW, K};
         s[n++] = {part + (int64_t)N * K, stride, nz, 1, N, db, N};
-        part += lin3::wgrad_floats(N, K);
+        part += lin3::wgrad_floats(rows, N, K);
         return GNN_OK;
     }
 };
-static int64_t tc_grad_floats(const gnn_mlp& P, int in, int sources) {
-    int64_t f = (int64_t)lin3::kMaxCtas * 2 * P.dims[P.n_lin] + sources * lin3::wgrad_floats(P.dims[1], in);
-    for (int k = 1; k < P.n_lin; ++k) f += lin3::wgrad_floats(P.dims[k + 1], P.dims[k]);
+// Partials of an MLP's backward over `rows` rows, and of the first Linear's `more` further sources over `more_rows`.
+static int64_t tc_grad_floats(const gnn_mlp& P, int in, int64_t rows, int more = 0, int64_t more_rows = 0) {
+    int64_t f = lin3::max_ctas(rows) * 2 * P.dims[P.n_lin] + lin3::wgrad_floats(rows, P.dims[1], in) +
+                more * lin3::wgrad_floats(more_rows, P.dims[1], in);
+    for (int k = 1; k < P.n_lin; ++k) f += lin3::wgrad_floats(rows, P.dims[k + 1], P.dims[k]);
     return f;
 }
 
@@ -858,7 +860,7 @@ static int tc_chain_bwd(const gnn_mlp& P, const gnn_mlp& dP, int64_t rows, float
         if ((rc = lin3::run(lin3::kLnAdjoint, a, s, &nz))) return rc;
         gs.s[gs.n++] = {gs.part, 2 * H, nz, 1, H, dP.gamma, H};
         gs.s[gs.n++] = {gs.part + H, 2 * H, nz, 1, H, dP.beta, H};
-        gs.part += (int64_t)lin3::kMaxCtas * 2 * H;
+        gs.part += lin3::max_ctas(rows) * 2 * H;
         g = g0;
     }
     float* next = g == g0 ? g1 : g0;
@@ -917,7 +919,7 @@ static void carve_tc(Carve& c, const gnn_graph_dev& G, const gnn_mp_config& cfg,
     b.da = c.take<float>(NR * H);
     b.dP = c.take<float>(NR * H);
     b.dQ = c.take<float>(NR * H);
-    b.part = c.take<float>(tc_grad_floats(W.edge, cfg.hidden, 3) + tc_grad_floats(W.node, cfg.hidden, 2));
+    b.part = c.take<float>(tc_grad_floats(W.edge, cfg.hidden, E, 2, NR) + tc_grad_floats(W.node, cfg.hidden, NR, 1, NR));
 }
 
 // Receivers, P|Q and the edge MLP up to the input of its last Linear.
@@ -1297,7 +1299,7 @@ static void carve_mlp(Carve& c, const gnn_mlp& P, int64_t rows, bool bwd, float*
     if (bwd) {
         *g0 = c.take<float>(rows * wmax);
         *g1 = c.take<float>(rows * wmax);
-        *part = c.take<float>(tc_widths(P, P.dims[0]) ? tc_grad_floats(P, P.dims[0], 1)
+        *part = c.take<float>(tc_widths(P, P.dims[0]) ? tc_grad_floats(P, P.dims[0], rows)
                                                       : (int64_t)partial_floats(P, rows));
         *dYf = c.take<float>(rows * P.dims[P.n_lin]);
     }
