@@ -24,7 +24,7 @@
 //   k_proj_bwd    dQ, dx_in += dP W1a + dQ W1b, dW1a, dW1b
 // Tiles are processed in chunks of at most kChunkTiles (fewer when the
 // caller's workspace is smaller) so that the scratch stays bounded; each
-// kernel's per-CTA partials are summed (CTA order) into dW right after it, so
+// kernel's per-CTA partials are summed (fixed order) into dW right after it, so
 // every gradient has a fixed summation order.
 
 #include <algorithm>

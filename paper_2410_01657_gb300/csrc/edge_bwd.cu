@@ -633,7 +633,7 @@ int edge_backward(const gnn_graph_dev& G, int H, const gnn_mp_params& W, const E
     A.mlp = mlp_dev(W.edge);
     A.eps = o.eps;
     A.act_rows = G.n_edge_tiles * 128;
-    // H = 32: four groups of one thread per row while their tiles fit (up to 4 Linears), else two of two
+    // H = 32: four groups of one thread per row while their tiles fit (up to 5 Linears), else two of two
     // threads per row
     if (H == 64) return launch<64, 2, 32>(G, A, tm_e, tm_de, tm_h, grid, s);
     if (H == 32)

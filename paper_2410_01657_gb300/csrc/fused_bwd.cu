@@ -840,9 +840,11 @@ int backward_h(const gnn_graph_dev& G, const gnn_mp_config& cfg, const gnn_mp_pa
                cudaStream_t s, const __nv_bfloat16* act) {
     using C = CfgB<H>;
     const int Le = W.edge.n_lin, Ln = W.node.n_lin;
-    GNN_REQUIRE(edge_backward_supported(H, Le) && node_bwd_tcols<H>(Ln) <= 512, GNN_EUNSUPPORTED,
-                "gnn_mp_backward: BF16 backward at H=%d supports at most %d Linear layers per MLP", H,
-                H == 64 ? 4 : 7);
+    auto deep = [](int n) { return edge_backward_supported(H, n) && node_bwd_tcols<H>(n) <= 512; };
+    int most = GNN_MAX_LIN;
+    while (most > 0 && !deep(most)) --most;
+    GNN_REQUIRE(Le <= most && Ln <= most, GNN_EUNSUPPORTED,
+                "gnn_mp_backward: BF16 backward at H=%d supports at most %d Linear layers per MLP", H, most);
     BwdWs w = carve_bwd(ws, G, H, Le, Ln, a_star == nullptr);
     GNN_REQUIRE(ws_bytes >= w.bytes, GNN_ENOMEM, "gnn_mp_backward: workspace too small");
     const int64_t NR = G.n_rows, E = G.n_edges;

@@ -158,7 +158,8 @@ __device__ __forceinline__ void flush_acc(uint32_t tmem, int N, int m_valid, int
 
 // Per-CTA weight-gradient partials: segment s of the result is rows x cols of
 // dst (leading dimension dst_ld), read from the partials at src_off with
-// leading dimension src_ld; k_reduce_grads sums the CTAs' partials in CTA order.
+// leading dimension src_ld; k_reduce_grads sums the CTAs' partials in a fixed order
+// (every eighth CTA by one warp, then the warps).
 struct RedSeg {
     float* dst;
     int dst_ld, rows, cols;

@@ -20,7 +20,7 @@
 //   k_bwd_chain2 / k_bwd_chain  k = L-2 .. 1 (the layer adjoint's per-Linear kernels)
 //   k_bwd_chain<INPUT> dX = dz_0 W_0 and dW_0 = dz_0^T X
 // Every gradient is a fixed-order sum (per thread in row order, per CTA in
-// warp and group order, then over the CTAs in CTA order).
+// warp and group order, then over the CTAs in a fixed order).
 
 #include <algorithm>
 
