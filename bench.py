@@ -277,16 +277,6 @@ def measured_traffic(workload: str, kernels: list, n_edges: int):
         return None
 
 
-def sgemm_flops_per_step(G, hidden: int, n_lin: int, layers: int) -> float:
-    """GEMM FLOPs of one step of the FP32 path's SIMT kernels, widths above 128 (forward, recompute, dgrad, wgrad)."""
-    E, N, Hh = G.n_edges, G.n_rows, hidden
-    def chain(rows, d0):
-        dims = [d0] + [Hh] * n_lin
-        return sum(2.0 * rows * dims[k] * dims[k + 1] for k in range(n_lin))
-    per_layer_fwd = chain(E, 3 * Hh) + chain(N, 2 * Hh)
-    return layers * per_layer_fwd * 4.0     # forward + recompute + dgrad + wgrad
-
-
 def algorithmic_flops_per_step(G, hidden: int, n_lin: int, layers: int, fwd_only: bool = False,
                                split: bool = True) -> float:
     """Tensor FLOPs one step of the layer stack must compute (Eq. 5a, 5e).
@@ -595,17 +585,6 @@ def time_e2e(net, G, u, t, steps, warmup, dev):
     return statistics.median(times), statistics.mean(times), h2d, 4, kernels
 
 
-def measure_fp32_peak():
-    """FP32 SIMT FMA throughput of this GPU, measured by the library's FMA kernel
-    (TFLOP/s, 2 FLOPs per FMA) and its SM count."""
-    import ctypes as C
-
-    from paper_2410_01657_gb300 import binding as B
-    tf, sms = C.c_double(), C.c_int32()
-    B.call("gnn_measure_fp32_fma", C.byref(tf), C.byref(sms), None)
-    return float(tf.value), int(sms.value)
-
-
 def fp32_comparison(dev, wl: dict, part_full, steps: int, warmup: int, ms_bf16_full: float):
     """The FP32 path against the fused BF16 path, same graph and step
     (eager steps, median). For the H=128 brick the comparison graph is the
@@ -615,16 +594,10 @@ def fp32_comparison(dev, wl: dict, part_full, steps: int, warmup: int, ms_bf16_f
     sub_nel = wl.get("fp32_nel")
     part = part_full if sub_nel is None else workload_graph(dict(wl, nel=sub_nel), sub_nel)[0]
     res = {}
-    sgemm = None
     for prec in ("bf16", "fp32"):
         G, _, stack, dx, _, _ = build_problem(dev, prec, wl, part)
         run = prepare_timing(stack, dx, 2, graph=False)
         res[prec] = statistics.median(time_steps(run, steps, torch.cuda.current_stream()))
-        if prec == "fp32":   # its SIMT GEMMs (widths above 128) against the measured FP32 FMA peak
-            rep = _profiled(run, 1)
-            n_lin = wl.get("nh", NH) + 2
-            if "k_sgemm" in rep:
-                sgemm = (sgemm_flops_per_step(G, wl["H"], n_lin, M), rep["k_sgemm"][1])
         del stack, G
         torch.cuda.empty_cache()
     L = (sub_nel or wl["nel"]) * wl["p"] + 1 if wl.get("mesh") != "mixed" else None
@@ -635,14 +608,6 @@ def fp32_comparison(dev, wl: dict, part_full, steps: int, warmup: int, ms_bf16_f
            f"{sub_nel}^3 elements p={wl['p']}, {wl['parts']} RCB sub-graphs ({L ** 3:,} nodes, {e_unpart:,} edges): "
            "the FP32 path keeps FP32 per-edge activations (35 GB per array at 32^3), which do not "
            "fit the full graph", "timing": "eager steps, median"}
-    tf, sms = measure_fp32_peak()
-    out["simt_peak"] = {"tflops": tf, "sm_count": sms,
-                        "src": "measured: the library's FP32 FMA kernel (gnn_measure_fp32_fma)"}
-    if sgemm is not None:
-        fl, ms_k = sgemm
-        out["sgemm"] = {"tflops": fl / (ms_k * 1e-3) / 1e12, "frac": fl / (ms_k * 1e-3) / 1e12 / tf,
-                        "ms_per_step": ms_k, "note": "the plain path's k_sgemm launches of one step (forward, "
-                                                     "recompute, input and weight gradients) over the SIMT peak"}
     return out
 
 
@@ -723,12 +688,6 @@ def main():
                                 "traffic": traffic.get(top_name) if traffic else None,
                                 "note": "bytes the kernel moves as designed (scratch and stored activations "
                                         "included), over its event-timed launches in profiled eager steps"})
-        elif top_name == "k_sgemm":   # the FP32 bench: the SIMT GEMMs against the measured FP32 FMA peak
-            tf, sms = measure_fp32_peak()
-            flops = sgemm_flops_per_step(G, Hw, n_lin, M)
-            ach = flops / (top_ms / n_prof * 1e-3) / 1e12
-            roof_kernel.update({"bound": "alu", "achieved": ach, "peak": tf, "unit": "TFLOP/s", "frac": ach / tf,
-                                "peak_src": f"measured: FP32 FMA kernel on {sms} SMs"})
 
     # the cost of consistency: the same stack with Eq. 5c-5d skipped (the paper's "None" layers)
     for c in (stack.cfg, stack.cfg_last):

@@ -19,10 +19,10 @@
 //                     for dgamma, dbeta, db_{L-1}
 //   k_bwd_chain2 / k_bwd_chain  k = L-1 .. 1: dz_{k-1} = (dz_k W_k) ELU'(h_{k-1}),
 //                     dW_k, db_{k-1} (the layer adjoint's per-Linear kernels)
-//   k_rowenc_w0       dW_0 = dz_0^T X, and dX = dz_0 W_0 when asked (db_0 comes
-//                     from the chain's last pass)
+//   k_rowenc_w0_rows  dW_0 = dz_0^T X (db_0 comes from the chain's last pass), or,
+//   k_rowenc_w0       when dX = dz_0 W_0 is asked for, both
 // Every gradient is a fixed-order sum: per thread in row order, per CTA in
-// warp order, then k_reduce_grads over the CTAs in CTA order.
+// warp order, then k_reduce_grads over the CTAs in a fixed order.
 
 #include <algorithm>
 
@@ -458,7 +458,7 @@ struct W0Args {
     const __nv_bfloat16* dz;   // dz_0 rows of the chunk, tile-padded [(t1 - t0) * 128 x 128]
     const float* X;            // [n_rows x K0]
     const float* W0;           // [128 x K0]
-    float* dX;                 // [n_rows x K0], NULL: not wanted
+    float* dX;                 // [n_rows x K0] (k_rowenc_w0)
     int64_t n_rows, t0, t1;
     int K0;
     float* part;               // per-CTA: dW_0 [128 x 16]
@@ -482,8 +482,7 @@ __global__ void __launch_bounds__(kW0NT) k_rowenc_w0(W0Args A) {
     float* sX = reinterpret_cast<float*>(w0_smem + W0Smem::x);
     float* sW = reinterpret_cast<float*>(w0_smem + W0Smem::w);
     const int tid = threadIdx.x, c = tid & (kH - 1), kh = tid >> 7, K0 = A.K0;
-    if (A.dX)
-        for (int i = tid; i < kH * kKP; i += kW0NT) sW[i] = (i % kKP) < K0 ? A.W0[(i / kKP) * K0 + i % kKP] : 0.f;
+    for (int i = tid; i < kH * kKP; i += kW0NT) sW[i] = (i % kKP) < K0 ? A.W0[(i / kKP) * K0 + i % kKP] : 0.f;
     float2 acc[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[j] = make_float2(0.f, 0.f);
@@ -511,7 +510,7 @@ __global__ void __launch_bounds__(kW0NT) k_rowenc_w0(W0Args A) {
             acc[2] = __ffma2_rn(d2, make_float2(x1.x, x1.y), acc[2]);
             acc[3] = __ffma2_rn(d2, make_float2(x1.z, x1.w), acc[3]);
         }
-        if (A.dX && rbase + c < A.n_rows) {   // thread (row = c, kh)
+        if (rbase + c < A.n_rows) {   // thread (row = c, kh)
             float2 o[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) o[j] = make_float2(0.f, 0.f);
